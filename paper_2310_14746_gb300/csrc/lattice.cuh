@@ -264,6 +264,21 @@ struct Phys {
     C Fx, Fy, Fz;  // body force
 };
 
+// FP64 kernels also take the uniform products of the collision from the host: per
+// opposite pair, in the order of its lower index, and per |c|^2.
+struct PairForce {
+    double G[9];          // 9 guo w (c.F)
+    double Q[9];          // g (c.F)
+    double H[9];          // (c.F) / 2
+    double F[9];          // c.F
+    double ow[3], gw[3];  // omega w, guo w of |c|^2 = 0, 1, 2
+};
+template <>
+struct Phys<double> {
+    double omega, guo, k1, k2, g1, g2, Fx, Fy, Fz;
+    PairForce pair;
+};
+
 // Coefficients k1 (|c|^2 = 1, na directions along an axis) and k2 (|c|^2 = 2,
 // nb of them touch an axis) with na*k1 + nb*k2 == target exactly (checked in
 // double for float; FP64 keeps the plain rounding, its bias is at 1e-16).
@@ -302,6 +317,27 @@ __host__ inline Phys<C> make_phys(double tau, const double F[3]) {
     p.Fx = C(F[0]);
     p.Fy = C(F[1]);
     p.Fz = Q == 9 ? C(0) : C(F[2]);
+    if constexpr (sizeof(C) == 8) {
+        int n = 0;
+        for (int i = 1; i < Q; ++i) {
+            if (opp<Q>(i) < i) continue;
+            // the +1 components, then the -1 components, in axis order (as the kernels add them)
+            double cF = 0.0;
+            cF += Lat<Q>::cx(i) * p.Fx;
+            cF += Lat<Q>::cy(i) * p.Fy;
+            cF += Lat<Q>::cz(i) * p.Fz;
+            const int c2 = Lat<Q>::cx(i) * Lat<Q>::cx(i) + Lat<Q>::cy(i) * Lat<Q>::cy(i) + Lat<Q>::cz(i) * Lat<Q>::cz(i);
+            p.pair.G[n] = 9.0 * p.guo * Lat<Q>::w(i) * cF;
+            p.pair.Q[n] = (c2 == 1 ? p.g1 : p.g2) * cF;
+            p.pair.H[n] = 0.5 * cF;
+            p.pair.F[n] = cF;
+            p.pair.ow[c2] = p.omega * Lat<Q>::w(i);
+            p.pair.gw[c2] = p.guo * Lat<Q>::w(i);
+            ++n;
+        }
+        p.pair.ow[0] = p.omega * Lat<Q>::w(0);
+        p.pair.gw[0] = p.guo * Lat<Q>::w(0);
+    }
     return p;
 }
 
@@ -569,6 +605,130 @@ __device__ __forceinline__ void for_pairs(F&& f) {
     }
 }
 
+// Position of a pair (by its lower index I) in the order of the lower indices.
+template <int Q>
+__host__ __device__ constexpr int pair_pos(int I) {
+    int n = 0;
+    for (int i = 1; i < I; ++i) n += opp<Q>(i) > i;
+    return n;
+}
+
+// Uniform products of the lane form for direction I. In FP64 they come from the
+// host (the FP64 pipe is the bound); in FP32 a thread forms them, which costs
+// less than holding them in registers.
+template <int Q, int I, class S>
+__device__ __forceinline__ S omega_w(const Phys<S>& ph) {
+    using L = Lat<Q>;
+    if constexpr (std::is_same_v<S, double>) return ph.pair.ow[L::cx(I) * L::cx(I) + L::cy(I) * L::cy(I) + L::cz(I) * L::cz(I)];
+    else return mul_(ph.omega, S(L::w(I)));
+}
+template <int Q, int I, class S>
+__device__ __forceinline__ S guo_w(const Phys<S>& ph, S guo_s) {
+    using L = Lat<Q>;
+    if constexpr (std::is_same_v<S, double>) return ph.pair.gw[L::cx(I) * L::cx(I) + L::cy(I) * L::cy(I) + L::cz(I) * L::cz(I)];
+    else return mul_(guo_s, S(L::w(I)));
+}
+template <int Q, int I, bool FX_ONLY, class S>
+__device__ __forceinline__ S c_force(const Phys<S>& ph) {  // c.F
+    if constexpr (std::is_same_v<S, double>) return ph.pair.F[pair_pos<Q>(I)];
+    else return FX_ONLY ? (Lat<Q>::cx(I) > 0 ? ph.Fx : -ph.Fx) : cdot_s<Q, I>(ph.Fx, ph.Fy, ph.Fz);
+}
+template <int Q, int I, class S>
+__device__ __forceinline__ S half_force(const Phys<S>& ph, S cF) {  // c.F / 2
+    if constexpr (std::is_same_v<S, double>) return ph.pair.H[pair_pos<Q>(I)];
+    else return mul_(S(0.5), cF);
+}
+template <int Q, int I, class S>
+__device__ __forceinline__ S guo_force(const Phys<S>& ph, S g, S cF) {  // g (c.F)
+    if constexpr (std::is_same_v<S, double>) return ph.pair.Q[pair_pos<Q>(I)];
+    else return mul_(g, cF);
+}
+
+// c.m over the pair differences m_I = d_I - d_opp(I): one axis of the momentum.
+template <int Q, int A>
+__device__ __forceinline__ double pair_axis_sum(const double* m) {
+    using L = Lat<Q>;
+    double r = 0.0;
+    for_pairs<Q>([&](auto ic) {
+        constexpr int I = decltype(ic)::value, n = pair_pos<Q>(I);
+        constexpr int first = 1 + 2 * A;  // the face direction of the axis (D3Q19)
+        if constexpr (I == first) r = m[n];
+    });
+    for_pairs<Q>([&](auto ic) {
+        constexpr int I = decltype(ic)::value, n = pair_pos<Q>(I);
+        constexpr int c = A == 0 ? L::cx(I) : (A == 1 ? L::cy(I) : L::cz(I));
+        constexpr int first = 1 + 2 * A;
+        if constexpr (I != first && c > 0) r = add_(r, m[n]);
+        if constexpr (I != first && c < 0) r = sub_(r, m[n]);
+    });
+    return r;
+}
+
+// The D3Q19 shift-form collision in FP64, arranged for the fewest FP64 operations: the
+// FP64 pipe (two lanes per clock and SM) bounds every FP64 kernel, not memory.
+// With the pair sums s = d_i + d_opp and differences m, t = omega A + guo (-3 u.F),
+// K = 4.5 omega rho varpi^2 and P = varpi rho k:
+//   even = w t + w K (c.u)^2 + G (c.u),  odd = P (c.u) + Q,
+//   d_i, d_opp <- (keep/2 s + even) +- (keep/2 m + odd),
+// since rho (c.u) = c.j + c.F/2 and c.v = varpi (c.u). About 145 operations per
+// D3Q19 cell with the force along x instead of about 200 in the lane form below
+// (whose order keeps the FP32 forms free of a rounding bias; in FP64 that bias
+// is of order 1e-16). Measured: D3Q19 160^3 1546 -> 1094 us per step, 110x90x100
+// with a general force 616 -> 356 us. D2Q9 keeps the order of the lane form, only
+// without its uniform products (the host forms them): the channel it validates
+// against the Brinkman profile has moments that vanish up to rounding (its
+// transverse momentum), and those follow the order of every operation.
+template <bool FX_ONLY, class Pop, class Sink>
+__device__ __forceinline__ void collide_shift64(const Pop& d, double varpi, const Phys<double>& ph, Sink out) {
+    constexpr int Q = 19, NP = 9;
+    using L = Lat<Q>;
+    double s[NP], m[NP];
+    for_pairs<Q>([&](auto ic) {
+        constexpr int I = decltype(ic)::value, J = opp<Q>(I), n = pair_pos<Q>(I);
+        s[n] = add_(d[I], d[J]);
+        m[n] = sub_(d[I], d[J]);
+    });
+    double drho = d[0];
+#pragma unroll
+    for (int n = 0; n < NP; ++n) drho = add_(drho, s[n]);
+    const double jx = pair_axis_sum<Q, 0>(m), jy = pair_axis_sum<Q, 1>(m), jz = pair_axis_sum<Q, 2>(m);
+    const double rho = add_(1.0, drho), inv = rcp_(rho), h = mul_(0.5, inv);
+    const double ux = fma_(ph.Fx, h, mul_(jx, inv));
+    const double uy = FX_ONLY ? mul_(jy, inv) : fma_(ph.Fy, h, mul_(jy, inv));
+    const double uz = FX_ONLY ? mul_(jz, inv) : fma_(ph.Fz, h, mul_(jz, inv));
+    const double x2 = mul_(ux, ux), y2 = mul_(uy, uy), z2 = mul_(uz, uz);
+    const double uu = add_(add_(x2, y2), z2);
+    const double vr = mul_(varpi, rho), v2r = mul_(varpi, vr);
+    const double A = fma_(mul_(-1.5, v2r), uu, drho);
+    double uF = mul_(ux, ph.Fx);
+    if (!FX_ONLY) uF = fma_(uz, ph.Fz, fma_(uy, ph.Fy, uF));
+    const double t = fma_(ph.omega, A, mul_(mul_(-3.0, ph.guo), uF));
+    const double K = mul_(mul_(4.5, ph.omega), v2r);
+    const double B1 = mul_(L::w(1), t), B2 = mul_(L::w(Q - 1), t);
+    const double K1 = mul_(L::w(1), K), K2 = mul_(L::w(Q - 1), K);
+    const double P1 = mul_(ph.k1, vr), P2 = mul_(ph.k2, vr);
+    const double keep = sub_(1.0, ph.omega), hk = mul_(0.5, keep);  // uniform
+    out(0, fma_(keep, d[0], mul_(L::w(0), t)));
+    for_pairs<Q>([&](auto ic) {
+        constexpr int I = decltype(ic)::value, J = opp<Q>(I), n = pair_pos<Q>(I);
+        constexpr int cx = L::cx(I), cy = L::cy(I), cz = L::cz(I), c2 = cx * cx + cy * cy + cz * cz;
+        constexpr bool forced = !FX_ONLY || cx != 0;
+        const double cu = c2 == 1 ? (cx ? ux : (cy ? uy : uz)) : cdot_i<Q, I>(ux, uy, uz);
+        const double B = c2 == 1 ? B1 : B2, Kw = c2 == 1 ? K1 : K2, P = c2 == 1 ? P1 : P2;
+        double even, odd;
+        if (forced) {
+            even = fma_(cu, fma_(Kw, cu, ph.pair.G[n]), B);
+            odd = fma_(hk, m[n], fma_(P, cu, ph.pair.Q[n]));
+        } else {
+            even = fma_(Kw, c2 == 1 ? (cx ? x2 : (cy ? y2 : z2)) : mul_(cu, cu), B);
+            odd = fma_(P, cu, mul_(hk, m[n]));
+        }
+        even = fma_(hk, s[n], even);
+        out(I, add_(even, odd));
+        out(J, sub_(even, odd));
+    });
+}
+
 // HBGK collision of one cell (or of two, V = F2), in place on the deviations d
 // (Sec. 3.2: relaxation toward the Maxwellian at varpi*u; Guo's source built
 // with u). Opposite directions share the even part of the equilibrium and of
@@ -584,13 +744,14 @@ __device__ __forceinline__ void for_pairs(F&& f) {
 // after rounding: products only feed multiplies and fmas. That keeps the paired
 // and the scalar evaluations bit-identical.
 template <int Q, class V, bool SCALED, bool FX_ONLY, class Pop, class Sink>
-__device__ __forceinline__ void collide(const Pop& d, V varpi, const Phys<typename Lane<V>::S>& ph,
-                                        typename Lane<V>::S s, typename Lane<V>::S inv_s, Sink out) {
+__device__ __forceinline__ void collide_lanes(const Pop& d, V varpi, const Phys<typename Lane<V>::S>& ph,
+                                              typename Lane<V>::S s, typename Lane<V>::S inv_s, Sink out) {
     // FX_ONLY: the caller guarantees F = (Fx, 0, 0); the terms with c.F = 0 drop out.
     // With SCALED the d are s * (f - w) on entry and exit; every term below
     // that adds into d carries the factor s (a power of two: exact).
     using L = Lat<Q>;
     using S = typename Lane<V>::S;
+    constexpr bool kLean = Q == 9 && std::is_same_v<V, double>;
     V drho_s, jxs, jys, jzs;  // sums in the units of d
     moments_x<Q, V>(d, drho_s, jxs, jys, jzs);
     const V rho = SCALED ? fma_(drho_s, V(inv_s), V(S(1))) : add_(V(S(1)), drho_s);
@@ -599,20 +760,21 @@ __device__ __forceinline__ void collide(const Pop& d, V varpi, const Phys<typena
     const V h = mul_(V(S(0.5)), inv_rho);
     const V ux = fma_(V(ph.Fx), h, mul_(jxs, im));
     const V uy = FX_ONLY ? mul_(jys, im) : fma_(V(ph.Fy), h, mul_(jys, im));
-    const V uz = FX_ONLY ? mul_(jzs, im) : fma_(V(ph.Fz), h, mul_(jzs, im));
+    const V uz = kLean ? V(S(0)) : FX_ONLY ? mul_(jzs, im) : fma_(V(ph.Fz), h, mul_(jzs, im));
     const V rho_s = SCALED ? mul_(rho, V(s)) : rho;
-    const V uu = fma_(uz, uz, fma_(uy, uy, mul_(ux, ux)));
+    // (D2Q9 in FP64: uz = 0 would cost FP64 operations that add nothing)
+    const V uu = kLean ? fma_(uy, uy, mul_(ux, ux)) : fma_(uz, uz, fma_(uy, uy, mul_(ux, ux)));
     const V vv = mul_(mul_(varpi, varpi), uu);
     const V A = fma_(mul_(rho_s, V(S(-1.5))), vv, drho_s);
     // -3 u.F
     const V nuF3 = FX_ONLY ? mul_(ux, V(mul_(S(-3), ph.Fx)))
-                           : mul_(V(S(-3)), fma_(uz, V(ph.Fz), fma_(uy, V(ph.Fy), mul_(ux, V(ph.Fx)))));
+                  : kLean ? mul_(V(S(-3)), fma_(uy, V(ph.Fy), mul_(ux, V(ph.Fx))))
+                          : mul_(V(S(-3)), fma_(uz, V(ph.Fz), fma_(uy, V(ph.Fy), mul_(ux, V(ph.Fx)))));
     const V r45 = mul_(V(S(4.5)), rho_s);
     const V keep = V(sub_(S(1), ph.omega));
     const S guo_s = SCALED ? mul_(ph.guo, s) : ph.guo;
     {  // rest population
-        const S w = S(L::w(0));
-        out(0, fma_(keep, V(d[0]), fma_(V(mul_(ph.omega, w)), A, mul_(V(mul_(guo_s, w)), nuF3))));
+        out(0, fma_(keep, V(d[0]), fma_(V(omega_w<Q, 0>(ph)), A, mul_(V(guo_w<Q, 0>(ph, guo_s)), nuF3))));
     }
     const V kv1 = mul_(V(ph.k1), varpi), kv2 = mul_(V(ph.k2), varpi);
     const S g1 = SCALED ? mul_(ph.g1, s) : ph.g1, g2 = SCALED ? mul_(ph.g2, s) : ph.g2;
@@ -620,8 +782,7 @@ __device__ __forceinline__ void collide(const Pop& d, V varpi, const Phys<typena
     for_pairs<Q>([&](auto ic) {
         constexpr int I = decltype(ic)::value;
         constexpr int c2 = L::cx(I) * L::cx(I) + L::cy(I) * L::cy(I) + L::cz(I) * L::cz(I);
-        const S w = S(L::w(I));
-        const V ow = V(mul_(ph.omega, w)), gw = V(mul_(guo_s, w));
+        const V ow = V(omega_w<Q, I>(ph)), gw = V(guo_w<Q, I>(ph, guo_s));
         const V cj = cdot_i<Q, I>(jxs, jys, jzs);  // c.j in the units of d
         const V kv = c2 == 1 ? kv1 : kv2;
         if (FX_ONLY && L::cx(I) == 0) {  // c.F = 0: the odd part is the product kv (c.j)
@@ -631,16 +792,23 @@ __device__ __forceinline__ void collide(const Pop& d, V varpi, const Phys<typena
             const V nkv = mul_(V(c2 == 1 ? -ph.k1 : -ph.k2), varpi);
             relax_pair_prod<Q, I>(d, keep, even, kv, nkv, cj, out);
         } else {
-            const S cF = FX_ONLY ? (L::cx(I) > 0 ? ph.Fx : -ph.Fx) : cdot_s<Q, I>(ph.Fx, ph.Fy, ph.Fz);
+            const S cF = c_force<Q, I, FX_ONLY>(ph);
             const V cu = fma_(V(cF), h, mul_(cj, im));
             const V cv = mul_(varpi, cu);
             const V kvs = c2 == 1 ? kvs1 : kvs2;
             const S g = c2 == 1 ? g1 : g2;
             const V even = fma_(ow, fma_(r45, mul_(cv, cv), A), mul_(gw, fma_(mul_(V(S(9)), cu), V(cF), nuF3)));
-            const V odd = fma_(kv, cj, fma_(kvs, V(mul_(S(0.5), cF)), V(mul_(g, cF))));
+            const V odd = fma_(kv, cj, fma_(kvs, V(half_force<Q, I>(ph, cF)), V(guo_force<Q, I>(ph, g, cF))));
             relax_pair<Q, I>(d, keep, even, odd, out);
         }
     });
+}
+
+template <int Q, class V, bool SCALED, bool FX_ONLY, class Pop, class Sink>
+__device__ __forceinline__ void collide(const Pop& d, V varpi, const Phys<typename Lane<V>::S>& ph,
+                                        typename Lane<V>::S s, typename Lane<V>::S inv_s, Sink out) {
+    if constexpr (std::is_same_v<V, double> && Q == 19) collide_shift64<FX_ONLY>(d, varpi, ph, out);
+    else collide_lanes<Q, V, SCALED, FX_ONLY>(d, varpi, ph, s, inv_s, out);
 }
 
 // Explicit-drag form of the homogenization (Sec. 3.3, eq. momentumHLBM): the
