@@ -29,6 +29,10 @@ int cuda_fail(cudaError_t e) {
     } while (0)
 
 constexpr int kGraphSteps = 8;  // even: a graph returns the state to its starting layout
+// Runs of a small lattice that one resident launch takes: below kResidentMin the launch and its
+// loads and stores (about 5 us) cost more than single steps; kResidentMax bounds one launch to
+// about a millisecond or two.
+constexpr long kResidentMin = 6, kResidentMax = 1000;
 
 // The lattice Layout enum values (lattice.cuh), repeated for host code.
 constexpr int kNatural = 0, kStreamed = 1, kSwapped = 2;
@@ -590,6 +594,14 @@ int hlbm_step(hlbm_t* h, long nsteps) {
     if (!h || nsteps < 0) return HLBM_ERR_INVALID_ARG;
     DeviceGuard g(h->device);
     long left = nsteps;
+    if (h->pattern == HLBM_TWO_LATTICE && left >= kResidentMin && resident_applies(h->ctx(h->stream))) {
+        while (left >= kResidentMin) {
+            const long n = left < kResidentMax ? left : kResidentMax;
+            HLBM_CUDA(launch_resident(h->ctx(h->stream), h->state(), h->varpi, (int)n));
+            left -= n;
+            h->step += n;
+        }
+    }
     while (left > 0) {
         if (left >= kGraphSteps && at_graph_origin(h)) {
             if (h->graph_dirty || !h->gexec) {

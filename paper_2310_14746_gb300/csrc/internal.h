@@ -38,6 +38,13 @@ cudaError_t launch_build_links(const LaunchCtx& c, const unsigned char* solid, u
 cudaError_t launch_step(const LaunchCtx& c, int mode, const void* fin, void* fout,
                         const float* varpi);
 
+// Many time steps of a small two-lattice state in one launch, in place on `f`
+// (NATURAL layout), with the state resident in the shared memory of one
+// thread-block cluster: the same bits as nsteps MODE_TWO_LATTICE steps.
+// resident_applies says whether the lattice fits (on the current device).
+bool resident_applies(const LaunchCtx& c);
+cudaError_t launch_resident(const LaunchCtx& c, void* f, const float* varpi, int nsteps);
+
 // Moments of a state stored in `layout` (Layout enum of lattice.cuh). rho
 // and/or u may be null. out_f64 selects double outputs, else float.
 cudaError_t launch_moments(const LaunchCtx& c, int layout, const void* f, void* rho, void* u,
