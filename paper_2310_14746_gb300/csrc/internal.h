@@ -27,6 +27,21 @@ struct LaunchCtx {
     int variant = 0;                 // 0: fastest applicable step kernel; 1: per-cell kernel only
 };
 
+// Block of a one-thread-per-cell kernel: a whole row of x as long as it fits 256
+// threads (at least 128 threads), a longer row in equal pieces where that leaves
+// fewer idle lanes than blocks of 128 cells times two rows, the only shape before:
+// those left up to 40 % of the lanes of a ragged row idle. Measured on the step,
+// 128-cell blocks vs this rule, us: FP32 150x101x67 with walls 32.1 -> 28.8, 160^3
+// with walls 113 -> 102, 221x143x203 163 -> 159, 256^3 376.6 -> 373.4, 128^3 49.4 ->
+// 49.5, 64^3 5.81 -> 5.46, 48^3 4.10 -> 3.84, 33x41x44 4.04 -> 3.33; FP16 152x104x96
+// with walls 41.2 -> 35.9. Equal pieces with as many idle lanes measured 4 % slower
+// (D2Q9 329x245), so a tie keeps the old shape.
+inline dim3 row_block(int nx) {
+    const int pieces = (nx + 255) / 256, bx = ((nx + pieces - 1) / pieces + 31) / 32 * 32;
+    if (pieces > 1 && pieces * bx >= (nx + 127) / 128 * 128) return dim3(128, 2, 1);
+    return dim3(bx, bx >= 128 ? 1 : 128 / bx, 1);
+}
+
 // Solid-link masks from a solid flag per cell (uint8, nonzero = solid): bit i of
 // links[cell] is set when the pull source x - c_i is solid (periodic wrap; a
 // source beyond a domain wall is left to the wall logic), bit 31 when the

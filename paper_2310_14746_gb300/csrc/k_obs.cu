@@ -8,6 +8,7 @@
 
 namespace hlbm {
 
+// Block of the reductions: their partition (and so the order of their sums) is part of the result.
 static dim3 block_for(int nx) {
     int bx = ((nx + 31) / 32) * 32;
     if (bx > 128) bx = 128;
@@ -63,7 +64,7 @@ template <int Q, class S, bool WALLS>
 static cudaError_t moments_impl(const LaunchCtx& c, int lay, const void* f, void* rho, void* u, int f64) {
     using C = typename S::C;
     const Geometry g = geom(c);
-    const dim3 blk = block_for(c.nx);
+    const dim3 blk = row_block(c.nx);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     const auto* a = static_cast<const typename S::T*>(f);
     if (f64)
@@ -293,7 +294,7 @@ k_fill_state(const double* fnat, int lay, Geometry g, typename S::C s, typename 
 template <int Q, class S, bool WALLS>
 static cudaError_t write_impl(const LaunchCtx& c, int lay, const double* fnat, int uniform, void* f) {
     using C = typename S::C;
-    const dim3 blk = block_for(c.nx);
+    const dim3 blk = row_block(c.nx);
     if (uniform) {
         const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, (c.nz + kFillZ - 1) / kFillZ);
         k_fill_state<Q, S, WALLS><<<grd, blk, 0, c.stream>>>(fnat, lay, geom(c), C(c.scale),
@@ -309,7 +310,7 @@ static cudaError_t write_impl(const LaunchCtx& c, int lay, const double* fnat, i
 template <int Q, class S, bool WALLS>
 static cudaError_t read_impl(const LaunchCtx& c, int lay, const void* f, double* fnat) {
     using C = typename S::C;
-    const dim3 blk = block_for(c.nx);
+    const dim3 blk = row_block(c.nx);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     k_read_state<Q, S, WALLS><<<grd, blk, 0, c.stream>>>(static_cast<const typename S::T*>(f), lay, geom(c),
                                                          C(1.0 / c.scale), fnat, c.links);

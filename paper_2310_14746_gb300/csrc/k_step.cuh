@@ -89,12 +89,6 @@ k_step(Planes<const typename S::T, Q> fin, Planes<typename S::T, Q> fout, const 
     for (int i = 0; i < Q; ++i) S::store_raw(scatter_ptr<Q, WALLS, lay_out>(fout, nb, cell, i), 0, d[i]);
 }
 
-inline dim3 step_block_for(int nx) {
-    int bx = ((nx + 31) / 32) * 32;
-    if (bx > 128) bx = 128;
-    return dim3(bx, 256 / bx, 1);
-}
-
 // FP64 blocks: one warp each, 32, 16 or 8 cells wide, whichever leaves the fewest
 // idle lanes (a warp instruction occupies the FP64 pipe for its 16 clocks however
 // many lanes are live, and the pipe bounds the step). One-warp blocks also spread
@@ -121,7 +115,7 @@ cudaError_t step_impl(const LaunchCtx& c, int mode, const void* fin, void* fout,
     using T = typename S::T;
     Geometry g{c.nx, c.ny, c.nz, c.wall[0], c.wall[1], c.wall[2], (size_t)c.nx * c.ny * c.nz};
     const Phys<C> ph = make_phys<C, Q>(c.tau, c.F);
-    const dim3 blk = S::kind == 0 ? step_block_f64(c.nx, c.ny) : step_block_for(c.nx);
+    const dim3 blk = S::kind == 0 ? step_block_f64(c.nx, c.ny) : row_block(c.nx);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     const C s = C(c.scale), inv_s = C(1.0 / c.scale);
     Planes<const T, Q> a;
