@@ -773,11 +773,15 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
     int rc = copy_natural(h, snaps, sc);
     if (rc != HLBM_OK) return rc;
 
-    // forward sweep, keeping f^{k*every}
+    // forward sweep, keeping f^{k*every}, and in the last segment every state: the reverse sweep
+    // starts there, so only the segments before it are recomputed (90 steps kept every 45: 134
+    // forward steps instead of 178). The final state goes to slot 0, which no segment uses.
+    const long last0 = (nsnap - 1) * every;
     void* a = snaps;
     for (long s = 0; s < nsteps; ++s) {
         const bool keep = (s + 1) % every == 0 && (s + 1) / every < nsnap;
-        void* b = keep ? (void*)(snaps + sb * ((s + 1) / every)) : (void*)(seg + sb * ((s + 1) & 1));
+        const long slot = s + 1 == nsteps ? 0 : (s >= last0 ? s + 1 - last0 : (s + 1) & 1);
+        void* b = keep ? (void*)(snaps + sb * ((s + 1) / every)) : (void*)(seg + sb * slot);
         HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, a, b, h->varpi));
         a = b;
     }
@@ -792,7 +796,8 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
         const long s0 = sg * every;
         const long s1 = s0 + every < nsteps ? s0 + every : nsteps;
         auto state = [&](long k) -> void* { return k == 0 ? (void*)(snaps + sb * sg) : (void*)(seg + sb * k); };
-        for (long k = 0; k + 1 < s1 - s0; ++k) HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, state(k), state(k + 1), h->varpi));
+        for (long k = 0; sg + 1 < nsnap && k + 1 < s1 - s0; ++k)
+            HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, state(k), state(k + 1), h->varpi));
         for (long s = s1 - 1; s >= s0; --s) {
             HLBM_CUDA(launch_adjoint_step(c, state(s - s0), lam_a, lam_b, h->varpi, gacc));
             float* t = lam_a;
