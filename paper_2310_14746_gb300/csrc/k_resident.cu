@@ -135,7 +135,9 @@ cudaError_t resident_impl(const LaunchCtx& c, const ResidentPlan& p, void* f, co
     using T = typename S::T;
     const auto kern = k_resident<Q, S, FORM, CELLS>;
     const int bytes = 2 * Q * p.chunk * (int)sizeof(T);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    // The limit is the kernel's largest size, not this launch's: several threads may launch it.
+    constexpr int kMaxBytes = 2 * Q * CELLS * kMaxThreads * (int)sizeof(T);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     const Geometry g{c.nx, c.ny, c.nz, c.wall[0], c.wall[1], c.wall[2], (size_t)c.nx * c.ny * c.nz};
