@@ -65,7 +65,9 @@ struct hlbm_lattice {
     cudaGraphExec_t gexec = nullptr;
     bool graph_dirty = true;
     int step_variant = HLBM_STEP_AUTO;
-    cudaMemPool_t pool = nullptr;  // scratch of the calls that need temporary device memory
+    cudaMemPool_t pool = nullptr;  // scratch, and the lattice of a handle that pool_keeps() all of
+    bool pooled = false;           // is this one?
+    bool moved = false;            // the stream was replaced: earlier work may be on another one
 
     size_t state_bytes() const { return (size_t)q * cells * storage_bytes(storage); }
     size_t arith_bytes() const { return storage == HLBM_F64 ? 8 : 4; }
@@ -97,21 +99,6 @@ struct hlbm_lattice {
 
 namespace {
 
-// All n values in [0, 1] (NaN fails)? The input may be a whole lattice (64 MiB
-// at 256^3), so the test runs in blocks without an early exit inside a block:
-// the inner loop vectorises, and a bad value still stops the scan at the end
-// of its block.
-bool host_unit_interval(const float* v, size_t n) {
-    constexpr size_t kBlock = 4096;
-    for (size_t b = 0; b < n; b += kBlock) {
-        const size_t e = b + kBlock < n ? b + kBlock : n;
-        int good = 1;
-        for (size_t k = b; k < e; ++k) good &= (v[k] >= 0.0f) & (v[k] <= 1.0f);
-        if (!good) return false;
-    }
-    return true;
-}
-
 // Make the handle's device current for the duration of a call.
 struct DeviceGuard {
     int prev = -1;
@@ -125,43 +112,38 @@ struct DeviceGuard {
 };
 
 // Temporary device memory of a call (the adjoint's checkpoints, staging buffers of host
-// I/O), stream-ordered on the handle's stream, from a memory pool private to the handle that
-// keeps what it has mapped for the next call. With the default pool (release threshold 0) the
-// 14.5 GB of checkpoints of a 128^3 x 2000-step gradient were unmapped at every
-// synchronisation and mapped again by the next call (0.395 s vs 0.370 s per gradient).
-// hlbm_release_scratch hands the memory back; hlbm_destroy destroys the pool.
+// I/O), stream-ordered on the handle's stream, from a pool that is the handle's own while
+// it lives and is kept for the next handle afterwards (mem.cu). It holds what it has
+// mapped: with the default pool (release threshold 0) the 14.5 GB of checkpoints of a
+// 128^3 x 2000-step gradient were unmapped at every synchronisation and mapped again by
+// the next call (0.395 s vs 0.370 s per gradient).
+// hlbm_release_scratch hands unused memory back.
 cudaError_t scratch_alloc(hlbm_t* h, void** p, size_t bytes) {
     if (!h->pool) {
-        cudaMemPoolProps pr;
-        std::memset(&pr, 0, sizeof(pr));
-        pr.allocType = cudaMemAllocationTypePinned;
-        pr.location.type = cudaMemLocationTypeDevice;
-        pr.location.id = h->device;
-        cudaError_t e = cudaMemPoolCreate(&h->pool, &pr);
-        if (e != cudaSuccess) {
-            h->pool = nullptr;
-            return e;
-        }
-        unsigned long long keep = ~0ull;  // never hand memory back on synchronisation
-        e = cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        const cudaError_t e = pool_acquire(&h->pool);
         if (e != cudaSuccess) return e;
     }
-    return cudaMallocFromPoolAsync(p, bytes, h->pool, h->stream);
+    return pool_alloc(h->pool, p, bytes, h->stream);
+}
+
+// Memory that stays for the handle's life. A small lattice takes it from the pool too:
+// the next one then finds it mapped. A large one would not be kept, and maps faster without
+// a pool (hlbm_create of a 384^3 FP16 lattice 2.7 ms, from a pool 5.9).
+cudaError_t lattice_alloc(hlbm_t* h, void** p, size_t bytes) {
+    return h->pooled ? scratch_alloc(h, p, bytes) : device_malloc(p, bytes);
 }
 
 void free_all(hlbm_t* h) {
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
-    cudaFree(h->buf[0]);
-    cudaFree(h->buf[1]);
-    cudaFree(h->varpi);
+    void* const blocks[] = {h->buf[0], h->buf[1], h->varpi, h->u_prev, h->partials, h->out8};
+    for (void* p : blocks)
+        if (p && (!h->pooled || cudaFreeAsync(p, h->stream) != cudaSuccess)) cudaFree(p);
     cudaFree(h->varpi3);
     cudaFree(h->links);
-    cudaFree(h->u_prev);
-    cudaFree(h->partials);
-    cudaFree(h->out8);
-    if (h->out8_host) cudaFreeHost(h->out8_host);
-    if (h->pool) cudaMemPoolDestroy(h->pool);  // every scratch block was freed on the stream
+    if (h->pool) cudaStreamSynchronize(h->stream);  // the pool may serve another stream next
+    slot_release(h->out8_host);
+    pool_release(h->pool);
 }
 
 // One direct time step on `s`, updating the bookkeeping.
@@ -299,13 +281,14 @@ int hlbm_create(hlbm_t** out, int velset, int nx, int ny, int nz, int storage, i
     h->scale = storage == HLBM_F16DEV ? 4096.0 : 1.0;
     cudaError_t e = cudaGetDevice(&h->device);
     const size_t nparts = reduce_partials_count(h->ctx(h->stream));
-    if (e == cudaSuccess) e = cudaMalloc(&h->buf[0], h->state_bytes());
-    if (e == cudaSuccess && pattern == HLBM_TWO_LATTICE) e = cudaMalloc(&h->buf[1], h->state_bytes());
-    if (e == cudaSuccess) e = cudaMalloc(&h->varpi, cells * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&h->u_prev, 3 * cells * h->arith_bytes());
-    if (e == cudaSuccess) e = cudaMalloc(&h->partials, nparts * 8 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&h->out8, 8 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMallocHost(&h->out8_host, 8 * sizeof(double));
+    h->pooled = pool_keeps((pattern == HLBM_TWO_LATTICE ? 2 : 1) * h->state_bytes() + cells * (sizeof(float) + 3 * h->arith_bytes()));
+    if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->buf[0], h->state_bytes());
+    if (e == cudaSuccess && pattern == HLBM_TWO_LATTICE) e = lattice_alloc(h, (void**)&h->buf[1], h->state_bytes());
+    if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->varpi, cells * sizeof(float));
+    if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->u_prev, 3 * cells * h->arith_bytes());
+    if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->partials, nparts * 8 * sizeof(double));
+    if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->out8, 8 * sizeof(double));
+    if (e == cudaSuccess && !(h->out8_host = slot_acquire())) e = cudaErrorMemoryAllocation;
     if (e == cudaSuccess) e = launch_fill_f32(h->varpi, cells, 1.0f, h->stream);
     if (e != cudaSuccess) {
         int rc = cuda_fail(e);
@@ -330,7 +313,8 @@ int hlbm_create(hlbm_t** out, int velset, int nx, int ny, int nz, int storage, i
 void hlbm_destroy(hlbm_t* h) {
     if (!h) return;
     DeviceGuard g(h->device);
-    cudaStreamSynchronize(h->stream);
+    if (h->moved) cudaDeviceSynchronize();
+    else cudaStreamSynchronize(h->stream);
     free_all(h);
     delete h;
 }
@@ -340,11 +324,13 @@ int hlbm_release_scratch(hlbm_t* h) {
     DeviceGuard g(h->device);
     HLBM_CUDA(cudaStreamSynchronize(h->stream));
     if (h->pool) HLBM_CUDA(cudaMemPoolTrimTo(h->pool, 0));
+    memory_give_back();
     return HLBM_OK;
 }
 
 int hlbm_set_stream(hlbm_t* h, void* cuda_stream) {
     if (!h) return HLBM_ERR_INVALID_ARG;
+    h->moved = h->moved || h->stream != static_cast<cudaStream_t>(cuda_stream);
     h->stream = static_cast<cudaStream_t>(cuda_stream);
     return HLBM_OK;
 }
@@ -498,7 +484,7 @@ int hlbm_set_solid_mask(hlbm_t* h, const unsigned char* solid, int on_device) {
     unsigned char* dsolid = nullptr;
     HLBM_CUDA(scratch_alloc(h, (void**)&tmp, (size_t)h->q * h->cells * sizeof(double)));
     cudaError_t e = launch_read_state(h->ctx(h->stream), h->layout(), h->state(), tmp);
-    if (e == cudaSuccess && !h->links) e = cudaMalloc(&h->links, h->cells * sizeof(unsigned));
+    if (e == cudaSuccess && !h->links) e = device_malloc((void**)&h->links, h->cells * sizeof(unsigned));
     if (e == cudaSuccess && !on_device) e = scratch_alloc(h, (void**)&dsolid, h->cells);
     if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(dsolid, solid, h->cells, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = launch_build_links(h->ctx(h->stream), on_device ? solid : dsolid, h->links);
@@ -516,7 +502,7 @@ int hlbm_set_porosity_tensor(hlbm_t* h, const float* varpi3, int on_device) {
     if (h->homog != HLBM_HOMOG_SHIFT) return HLBM_ERR_STATE;
     DeviceGuard g(h->device);
     const size_t n = 3 * h->cells;
-    if (!h->varpi3) HLBM_CUDA(cudaMalloc(&h->varpi3, n * sizeof(float)));
+    if (!h->varpi3) HLBM_CUDA(device_malloc((void**)&h->varpi3, n * sizeof(float)));
     if (!on_device) {
         if (!host_unit_interval(varpi3, n)) return HLBM_ERR_INVALID_ARG;
         HLBM_CUDA(cudaMemcpyAsync(h->varpi3, varpi3, n * sizeof(float), cudaMemcpyHostToDevice, h->stream));

@@ -91,6 +91,35 @@ cudaError_t launch_fill_bytes0(void* p, size_t bytes, cudaStream_t s);
 
 size_t storage_bytes(int storage);
 
+// Memory kept between objects, on the current device (mem.cu). A pool belongs to one handle at
+// a time; every block taken from it is freed, and its streams are drained, before it is released.
+bool pool_keeps(size_t bytes);  // does a released pool keep this much mapped?
+cudaError_t pool_acquire(cudaMemPool_t* pool);
+void pool_release(cudaMemPool_t pool);
+cudaError_t pool_shared(cudaMemPool_t* pool);  // the servers' pool
+cudaError_t pool_alloc(cudaMemPool_t pool, void** p, size_t bytes, cudaStream_t s);
+cudaError_t device_malloc(void** p, size_t bytes);  // cudaMalloc, for blocks that no pool should hold
+void* pinned_acquire(size_t bytes, size_t* capacity);  // null: out of memory
+void pinned_release(void* b, size_t capacity);
+double* slot_acquire();  // 64 bytes of pinned memory, or null
+void slot_release(double* p);
+void memory_give_back();  // return what is kept for later objects
+
+// All n values in [0, 1] (NaN fails)? The input may be a whole lattice (64 MiB
+// at 256^3), so the test runs in blocks without an early exit inside a block:
+// the inner loop vectorises, and a bad value still stops the scan at the end
+// of its block.
+inline bool host_unit_interval(const float* v, size_t n) {
+    constexpr size_t kBlock = 4096;
+    for (size_t b = 0; b < n; b += kBlock) {
+        const size_t e = b + kBlock < n ? b + kBlock : n;
+        int good = 1;
+        for (size_t k = b; k < e; ++k) good &= (v[k] >= 0.0f) & (v[k] <= 1.0f);
+        if (!good) return false;
+    }
+    return true;
+}
+
 // Reverse step of the outflow-flux adjoint: fn is the forward state before the
 // step (NATURAL layout), lam_in = dJ/df^{n+1} and lam_out = dJ/df^n ([q][cells]
 // FP32, distinct buffers); grad (FP32 cells) accumulates dJ/dvarpi.

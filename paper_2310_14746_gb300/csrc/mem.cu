@@ -1,0 +1,252 @@
+// Device and pinned host memory of handles and servers, kept between objects.
+//
+// Creating a lattice took about 0.4 ms, destroying it 0.3 to 1 ms, and the first
+// call that needs scratch mapped it again (1.4 ms for a 48^3 gradient over 90
+// steps, whose kernels run 1.6 ms): a design loop or a batch of small solves pays
+// that for every object. A handle therefore takes its scratch, and its lattice if
+// that is small, from a private stream-ordered pool, and a pool that is given back
+// is kept for the next handle on that device, trimmed to kKeepBytes; at most kKeepPools
+// are kept per device, the others are destroyed. Servers share one pool per device that
+// holds up to kKeepBytes unused (a slot's memory was mapped at each admission). Pinned
+// blocks are kept likewise, up to kKeepPinned bytes per device. A failed allocation first
+// returns what is kept. Nothing outlives the context it belongs to: what a device keeps is
+// forgotten when the context's id has changed. Measured: gradient of a 48^3 box over
+// 90 steps through torch.autograd, handle included, 3.52 -> 2.09 ms; submitting a 96^3
+// request 1.2 -> 0.34 ms.
+#include <cuda_runtime.h>
+
+#include <cstring>
+#include <map>
+#include <mutex>
+#include <vector>
+
+#include "internal.h"
+
+namespace hlbm {
+
+namespace {
+
+constexpr int kMaxDevices = 64;
+constexpr size_t kKeepPools = 2, kKeepBytes = (size_t)512 << 20;  // per device: at most 1.5 GiB stays mapped
+constexpr size_t kKeepPinned = (size_t)64 << 20;          // per device
+constexpr size_t kSlotBytes = 64, kSlots = 256;  // small pinned results (one page-locked block per device)
+
+struct Kept {
+    unsigned long long context = 0;  // id of the context that all of this belongs to
+    std::vector<cudaMemPool_t> pools;
+    cudaMemPool_t shared = nullptr;
+    std::multimap<size_t, void*> pinned;  // capacity -> block
+    size_t pinned_bytes = 0;
+    char* slots = nullptr;
+    std::vector<int> free_slots;
+};
+std::mutex& kept_mutex() {
+    static std::mutex* m = new std::mutex();
+    return *m;
+}
+
+// 0: no context is current.
+unsigned long long context_id() {
+    using GetId = int (*)(void*, unsigned long long*);
+    static const GetId get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &r) != cudaSuccess) f = nullptr;
+        return reinterpret_cast<GetId>(f);
+    }();
+    unsigned long long id = 0;
+    if (get && get(nullptr, &id) == 0) return id;
+    if (get && cudaFree(nullptr) == cudaSuccess && get(nullptr, &id) == 0) return id;  // creates the context
+    (void)cudaGetLastError();
+    return 0;
+}
+
+// What the current device keeps, under kept_mutex(). Null: nothing can be kept.
+// Never destroyed: objects may be released while the process ends.
+Kept* kept() {
+    static Kept* const all = new Kept[kMaxDevices];
+    int device = -1;
+    if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= kMaxDevices) return nullptr;
+    const unsigned long long id = context_id();
+    if (!id) return nullptr;
+    if (all[device].context != id) {
+        all[device] = Kept();
+        all[device].context = id;
+    }
+    return &all[device];
+}
+
+cudaError_t create_pool(unsigned long long hold, cudaMemPool_t* pool) {
+    *pool = nullptr;
+    cudaMemPoolProps pr;
+    std::memset(&pr, 0, sizeof(pr));
+    pr.allocType = cudaMemAllocationTypePinned;
+    pr.location.type = cudaMemLocationTypeDevice;
+    cudaError_t e = cudaGetDevice(&pr.location.id);
+    if (e != cudaSuccess) return e;
+    e = cudaMemPoolCreate(pool, &pr);
+    if (e == cudaSuccess) {
+        e = cudaMemPoolSetAttribute(*pool, cudaMemPoolAttrReleaseThreshold, &hold);
+        if (e != cudaSuccess) cudaMemPoolDestroy(*pool);
+    }
+    if (e != cudaSuccess) *pool = nullptr;
+    return e;
+}
+
+}  // namespace
+
+// All functions here work on the current device.
+
+void memory_give_back() {
+    std::vector<cudaMemPool_t> pools;
+    std::multimap<size_t, void*> blocks;
+    cudaMemPool_t shared = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        if (Kept* const k = kept()) {
+            pools.swap(k->pools);
+            blocks.swap(k->pinned);
+            k->pinned_bytes = 0;
+            shared = k->shared;
+        }
+    }
+    for (cudaMemPool_t p : pools) cudaMemPoolDestroy(p);
+    if (shared) cudaMemPoolTrimTo(shared, 0);
+    for (auto& b : blocks) cudaFreeHost(b.second);
+}
+
+bool pool_keeps(size_t bytes) { return bytes <= kKeepBytes; }
+
+cudaError_t pool_acquire(cudaMemPool_t* pool) {
+    {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        Kept* const k = kept();
+        if (k && !k->pools.empty()) {
+            *pool = k->pools.back();
+            k->pools.pop_back();
+            return cudaSuccess;
+        }
+    }
+    return create_pool(~0ull, pool);  // hands nothing back on synchronisation
+}
+
+cudaError_t pool_shared(cudaMemPool_t* pool) {
+    *pool = nullptr;
+    std::lock_guard<std::mutex> lk(kept_mutex());
+    Kept* const k = kept();
+    if (!k) return cudaErrorInvalidDevice;
+    if (!k->shared) {
+        const cudaError_t e = create_pool(kKeepBytes, &k->shared);
+        if (e != cudaSuccess) return e;
+    }
+    *pool = k->shared;
+    return cudaSuccess;
+}
+
+void pool_release(cudaMemPool_t pool) {
+    if (!pool) return;
+    if (cudaMemPoolTrimTo(pool, kKeepBytes) == cudaSuccess) {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        Kept* const k = kept();
+        if (k && k->pools.size() < kKeepPools) {
+            k->pools.push_back(pool);
+            return;
+        }
+    }
+    cudaMemPoolDestroy(pool);
+}
+
+cudaError_t pool_alloc(cudaMemPool_t pool, void** p, size_t bytes, cudaStream_t s) {
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        memory_give_back();
+        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    }
+    return e;
+}
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        memory_give_back();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
+void* pinned_acquire(size_t bytes, size_t* capacity) {
+    {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        if (Kept* const k = kept()) {
+            const auto it = k->pinned.lower_bound(bytes);
+            if (it != k->pinned.end() && it->first <= 2 * bytes) {
+                void* b = it->second;
+                *capacity = it->first;
+                k->pinned_bytes -= it->first;
+                k->pinned.erase(it);
+                return b;
+            }
+        }
+    }
+    void* b = nullptr;
+    *capacity = bytes;
+    if (cudaMallocHost(&b, bytes) == cudaSuccess) return b;
+    (void)cudaGetLastError();
+    memory_give_back();
+    if (cudaMallocHost(&b, bytes) == cudaSuccess) return b;
+    (void)cudaGetLastError();
+    return nullptr;
+}
+
+void pinned_release(void* b, size_t capacity) {
+    if (!b) return;
+    {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        Kept* const k = kept();
+        if (k && k->pinned_bytes + capacity <= kKeepPinned) {
+            k->pinned.emplace(capacity, b);
+            k->pinned_bytes += capacity;
+            return;
+        }
+    }
+    cudaFreeHost(b);
+}
+
+// 64 bytes of pinned memory.
+double* slot_acquire() {
+    void* b = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        Kept* const k = kept();
+        if (k && !k->slots && cudaHostAlloc(&b, kSlotBytes * kSlots, cudaHostAllocPortable) == cudaSuccess) {
+            k->slots = static_cast<char*>(b);
+            for (int i = (int)kSlots - 1; i >= 0; --i) k->free_slots.push_back(i);
+        }
+        if (k && !k->free_slots.empty()) {
+            const int i = k->free_slots.back();
+            k->free_slots.pop_back();
+            return reinterpret_cast<double*>(k->slots + (size_t)i * kSlotBytes);
+        }
+    }
+    if (cudaMallocHost(&b, kSlotBytes) == cudaSuccess) return static_cast<double*>(b);
+    (void)cudaGetLastError();
+    return nullptr;
+}
+
+void slot_release(double* p) {
+    if (!p) return;
+    char* const c = reinterpret_cast<char*>(p);
+    {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        Kept* const k = kept();
+        if (k && k->slots && c >= k->slots && c < k->slots + kSlotBytes * kSlots) {
+            k->free_slots.push_back((int)((c - k->slots) / kSlotBytes));
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
+}  // namespace hlbm

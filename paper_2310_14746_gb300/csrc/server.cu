@@ -380,6 +380,7 @@ struct Pending {
     uint64_t id;
     hlbm_request req;
     float* field = nullptr;  // pinned host copy of varpi
+    size_t field_bytes = 0;  // capacity of its block
     double t_submit = 0.0;
     int alloc_failures = 0;  // admissions that failed for lack of device memory
 };
@@ -427,6 +428,7 @@ struct hlbm_server {
     cudaStream_t branch[kGraphBranches] = {};  // capture streams of the graph's parallel branches
     cudaEvent_t fork_ev = nullptr, join_ev[kGraphBranches] = {};
     int device = 0;
+    cudaMemPool_t pool = nullptr;  // device memory of the slots: the servers' pool (mem.cu)
     std::mutex mu;
     std::deque<Pending> waiting;
     std::vector<Live> live;
@@ -442,6 +444,7 @@ struct hlbm_server {
     size_t partial_cap = 0;  // tiles
     double* dout = nullptr;
     double* hout = nullptr;
+    size_t htab_bytes = 0, hout_bytes = 0;  // capacities of the pinned blocks
     double* dfeq = nullptr;
     uint64_t next_id = 1;
     std::chrono::steady_clock::time_point t0;
@@ -523,7 +526,7 @@ void finish_pending(hlbm_server_t* s, Pending& p, int status) {
     r.t_admit = -1.0;
     r.t_finish = s->now();
     s->done.push_back(r);
-    cudaFreeHost(p.field);
+    pinned_release(p.field, p.field_bytes);
     p.field = nullptr;
 }
 
@@ -532,7 +535,7 @@ cudaError_t alloc_or_inject(hlbm_server_t* s, void** p, size_t bytes) {
         --s->inject_alloc_failures;
         return cudaErrorMemoryAllocation;
     }
-    return cudaMallocAsync(p, bytes, s->stream);
+    return pool_alloc(s->pool, p, bytes, s->stream);
 }
 
 // Allocate and initialise a slot; returns cudaSuccess or the failing error (nothing leaked).
@@ -772,7 +775,7 @@ int upload_table(hlbm_server_t* s) {
         s->dpartials = nullptr;
         s->partial_cap = 0;
         size_t cap = std::max<size_t>((size_t)tiles * 2, 4096);
-        SRV_CUDA(cudaMallocAsync(&s->dpartials, cap * 8 * sizeof(double), s->stream));
+        SRV_CUDA(pool_alloc(s->pool, (void**)&s->dpartials, cap * 8 * sizeof(double), s->stream));
         s->partial_cap = cap;
     }
     const size_t bytes = offsetof(DevTable, slot) + sizeof(DevSlot) * s->run.size();
@@ -816,10 +819,11 @@ int hlbm_server_create(hlbm_server_t** out, size_t mem_budget, int storage, int 
     double feq[19];
     for (int i = 0; i < 19; ++i) feq[i] = feq_rest(i);
     cudaError_t e = cudaGetDevice(&s->device);
+    if (e == cudaSuccess) e = pool_shared(&s->pool);
     if (e == cudaSuccess) e = cudaMalloc(&s->dtab, sizeof(DevTable));
-    if (e == cudaSuccess) e = cudaMallocHost(&s->htab, sizeof(DevTable));
+    if (e == cudaSuccess && !(s->htab = static_cast<DevTable*>(pinned_acquire(sizeof(DevTable), &s->htab_bytes)))) e = cudaErrorMemoryAllocation;
     if (e == cudaSuccess) e = cudaMalloc(&s->dout, kMaxSlots * 8 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMallocHost(&s->hout, kMaxSlots * 8 * sizeof(double));
+    if (e == cudaSuccess && !(s->hout = static_cast<double*>(pinned_acquire(kMaxSlots * 8 * sizeof(double), &s->hout_bytes)))) e = cudaErrorMemoryAllocation;
     if (e == cudaSuccess) e = cudaMalloc(&s->dfeq, sizeof(feq));
     if (e == cudaSuccess) e = cudaMemcpy(s->dfeq, feq, sizeof(feq), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
@@ -855,9 +859,9 @@ void hlbm_server_destroy(hlbm_server_t* s) {
     cudaStreamSynchronize(s->stream);
     for (Live& l : s->live) {
         free_slot(s, l);
-        cudaFreeHost(l.p.field);
+        pinned_release(l.p.field, l.p.field_bytes);
     }
-    for (Pending& p : s->waiting) cudaFreeHost(p.field);
+    for (Pending& p : s->waiting) pinned_release(p.field, p.field_bytes);
     if (s->dpartials) cudaFreeAsync(s->dpartials, s->stream);
     cudaStreamSynchronize(s->stream);
     if (s->gexec) cudaGraphExecDestroy(s->gexec);
@@ -870,8 +874,8 @@ void hlbm_server_destroy(hlbm_server_t* s) {
     cudaFree(s->dtab);
     cudaFree(s->dout);
     cudaFree(s->dfeq);
-    if (s->htab) cudaFreeHost(s->htab);
-    if (s->hout) cudaFreeHost(s->hout);
+    pinned_release(s->htab, s->htab_bytes);
+    pinned_release(s->hout, s->hout_bytes);
     delete s;
 }
 
@@ -883,12 +887,12 @@ int hlbm_server_submit(hlbm_server_t* s, const hlbm_request* r, uint64_t* id) {
     if (!(r->tol > 0.0) || r->max_steps < 1) return HLBM_ERR_INVALID_ARG;
     const size_t n = (size_t)r->nx * r->ny * r->nz;
     if (n > ((size_t)1 << 31) / 19) return HLBM_ERR_INVALID_ARG;
-    for (size_t k = 0; k < n; ++k)
-        if (!(r->varpi[k] >= 0.0f && r->varpi[k] <= 1.0f)) return HLBM_ERR_INVALID_ARG;
+    if (!host_unit_interval(r->varpi, n)) return HLBM_ERR_INVALID_ARG;
     if (s->slot_bytes(*r) > s->budget) return HLBM_ERR_OOM;
     Pending p;
     p.req = *r;
-    if (cudaMallocHost(&p.field, n * sizeof(float)) != cudaSuccess) return HLBM_ERR_OOM;
+    p.field = static_cast<float*>(pinned_acquire(n * sizeof(float), &p.field_bytes));
+    if (!p.field) return HLBM_ERR_OOM;
     std::memcpy(p.field, r->varpi, n * sizeof(float));
     p.req.varpi = nullptr;
     std::lock_guard<std::mutex> lk(s->mu);
@@ -969,7 +973,7 @@ int hlbm_server_pump(hlbm_server_t* s, int* active, int* waiting) {
             if (l.p.req.u_out && status != HLBM_ERR_CANCELLED) {
                 const size_t n = (size_t)l.ds.nx * l.ds.ny * l.ds.nz;
                 void* du = nullptr;
-                cudaError_t e = cudaMallocAsync(&du, 3 * n * sizeof(float), s->stream);
+                cudaError_t e = pool_alloc(s->pool, &du, 3 * n * sizeof(float), s->stream);
                 if (e == cudaSuccess) e = launch_moments(s->ctx_for(l), 0, l.ds.f[0], nullptr, du, 0);
                 if (e == cudaSuccess)
                     e = cudaMemcpyAsync(l.p.req.u_out, du, 3 * n * sizeof(float), cudaMemcpyDeviceToHost, s->stream);
@@ -979,7 +983,7 @@ int hlbm_server_pump(hlbm_server_t* s, int* active, int* waiting) {
             }
             finish(s, l, status, o);
             free_slot(s, l);
-            cudaFreeHost(l.p.field);
+            pinned_release(l.p.field, l.p.field_bytes);
             gone[i] = 1;
             s->table_dirty = true;
             return HLBM_OK;
