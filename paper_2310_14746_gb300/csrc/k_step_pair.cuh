@@ -58,24 +58,34 @@ struct Pair16<StoreBF16> {
     }
 };
 
-// Block width in threads (cell pairs) along x: 64 when it divides the row's
-// pair count, else 32, else the width (up to 128) that leaves the fewest idle
-// threads; short rows take the next power of two.
-inline int pair_block_x(int nx) {
-    const int pairs = nx / 2;
-    if (pairs <= 32) {
-        int b = 1;
-        while (b < pairs) b <<= 1;
-        return b;
-    }
-    if (pairs % 64 == 0) return 64;
-    if (pairs % 32 == 0) return 32;
-    int best = 64, waste_best = 1 << 30;
-    for (int b : {64, 32, 128, 96}) {
-        const int waste = ((pairs + b - 1) / b) * b - pairs;
-        if (waste < waste_best) {
-            best = b;
-            waste_best = waste;
+// Block of a paired kernel (x in cell pairs): about 128 threads that leave the fewest
+// idle lanes over the lattice, counting the row tail, the partly filled warp of a
+// block and the tail of y. Candidate widths: 64, 32 and 16 pairs, and the row cut into
+// one to four equal pieces (any width: a warp may span rows). Before, blocks had 256
+// threads and widths of 32, 64, 96 or 128 pairs. Measured, us per step before -> with
+// this rule: two-lattice FP16 96^3 15.4 -> 12.0, 160^3 63.1 -> 55.8, 42x50x60 4.35 ->
+// 3.59, 64^3 5.12 -> 4.61, 192^3 94.5 -> 92.8, 256^3 216.3 -> 214.1, 384x192x192 184.4 ->
+// 182.0; BF16 160^3 57.3 -> 53.2, 176x176x152 (drag) 70.9 -> 67.8, 204x190x180 (tensor)
+// 131 -> 126; in place FP16 80x64x72 8.7 -> 6.2, 160^3 63.7 -> 57.6, BF16 192^3 95.5 ->
+// 93.8. Pieces of 16 pairs where nx is no multiple of 32 measured 110 instead of 91.8
+// (BF16 222x144x200), hence the penalty.
+inline dim3 pair_block(int nx, int ny, int cap) {
+    const int pairs = nx / 2, most = cap < 192 ? cap : 192;
+    const int widths[] = {64, 32, 16, pairs, (pairs + 1) / 2, (pairs + 2) / 3, (pairs + 3) / 4};
+    dim3 best(32, 4, 1);
+    double score_best = -1.0;
+    for (int bx : widths) {
+        if (bx < 1 || bx > most) continue;
+        for (int by = 1; bx * by <= most; ++by) {
+            const int threads = bx * by, lanes = (threads + 31) / 32 * 32;
+            double score = (double)pairs / ((pairs + bx - 1) / bx) * by / lanes * ny / ((ny + by - 1) / by * by);
+            if (threads < 64) score *= 0.8;            // too few warps per block to fill an SM
+            if (bx < 32 && bx < pairs) score *= nx % 32 == 0 ? 0.97 : 0.85;  // short pieces, worse when they straddle lines
+            score -= 1e-4 * (threads < 128 ? 128 - threads : threads - 128) / 128;
+            if (score > score_best) {
+                score_best = score;
+                best = dim3(bx, by, 1);
+            }
         }
     }
     return best;
@@ -221,8 +231,8 @@ struct PairTraits {
 // resident warps per SM; measured at 384^3: 0.973 vs 0.955 of the copy
 // bandwidth at 64 registers). The FP16 kernel (whose unpack costs more
 // registers) and the in-place steps measured slower at 56 (FP16 0.919 vs 0.922,
-// AA 0.855 / 0.892 vs 0.884 / 0.912), so they keep 256-thread blocks and the
-// budget of PairTraits.
+// AA 0.855 / 0.892 vs 0.884 / 0.912), so they keep the budget of PairTraits, which
+// is stated for 256 threads (pair_block takes fewer).
 template <class S, int FORM, int MODE>
 struct PairLaunch {
     static constexpr bool k56 = S::kind == 3 /* BF16 */ && FORM == FORM_SHIFT_FX && MODE == MODE_TWO_LATTICE;
@@ -304,10 +314,8 @@ cudaError_t step_pair_impl(const LaunchCtx& c, const void* fin, void* fout, cons
     Geometry g{c.nx, c.ny, c.nz, 0, 0, 0, (size_t)c.nx * c.ny * c.nz};
     const Phys<float> ph = make_phys<float, Q>(c.tau, c.F);
     constexpr int threads = PairLaunch<S, FORM, MODE>::kThreads;
-    const int bx = pair_block_x(c.nx);
-    const int by = bx >= threads ? 1 : threads / bx;
-    const dim3 blk(bx, by, 1);
-    const dim3 grd((c.nx / 2 + bx - 1) / bx, (c.ny + by - 1) / by, c.nz);
+    const dim3 blk = pair_block(c.nx, c.ny, threads);
+    const dim3 grd((c.nx / 2 + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     Planes<const T, Q> a;
     Planes<T, Q> b;
     for (int i = 0; i < Q; ++i) {
