@@ -33,6 +33,12 @@ constexpr int kGraphSteps = 8;  // even: a graph returns the state to its starti
 // loads and stores (about 5 us) cost more than single steps; kResidentMax bounds one launch to
 // about a millisecond or two.
 constexpr long kResidentMin = 6, kResidentMax = 1000;
+// Samples of hlbm_reduce_series per graph replay. Even, so that a replay returns the state to its
+// starting layout. Launched one by one, the three kernels of a sample leave the GPU idle for about
+// a third of a 64^3 sample (step 5.5, diagnostics 9 us). A series of 200 samples, us: 24^3
+// 3290 -> 2210, 48^3 3700 -> 2670, 64^3 4400 -> 3180, 128^3 21260 -> 19980.
+constexpr int kSeriesSamples = 8;
+constexpr long kSeriesMin = 32;  // shorter series do not pay for the capture
 
 // The lattice Layout enum values (lattice.cuh), repeated for host code.
 constexpr int kNatural = 0, kStreamed = 1, kSwapped = 2;
@@ -64,6 +70,12 @@ struct hlbm_lattice {
     double* out8_host = nullptr;
     cudaGraphExec_t gexec = nullptr;
     bool graph_dirty = true;
+    cudaGraphExec_t series_exec = nullptr;  // kSeriesSamples samples of hlbm_reduce_series
+    int series_every = 0;                   // steps between its samples; 0: to be captured again
+    void settings_changed() {
+        graph_dirty = true;
+        series_every = 0;
+    }
     int step_variant = HLBM_STEP_AUTO;
     cudaMemPool_t pool = nullptr;  // scratch, and the lattice of a handle that pool_keeps() all of
     bool pooled = false;           // is this one?
@@ -135,6 +147,7 @@ cudaError_t lattice_alloc(hlbm_t* h, void** p, size_t bytes) {
 
 void free_all(hlbm_t* h) {
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
+    if (h->series_exec) cudaGraphExecDestroy(h->series_exec);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     void* const blocks[] = {h->buf[0], h->buf[1], h->varpi, h->u_prev, h->partials, h->out8};
     for (void* p : blocks)
@@ -161,14 +174,15 @@ int step_once(hlbm_t* h, cudaStream_t s) {
 
 bool at_graph_origin(const hlbm_t* h) { return h->pattern == HLBM_TWO_LATTICE ? h->cur == 0 : h->aa_odd == 0; }
 
-// Capture kGraphSteps steps starting from the graph origin layout.
-int build_graph(hlbm_t* h) {
+// Capture what `body` launches on the handle's capture stream, starting from the graph origin layout,
+// which an even number of steps returns to.
+template <class Body>
+int capture(hlbm_t* h, cudaGraphExec_t* exec, Body&& body) {
     if (!h->cap_stream) HLBM_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     const int cur0 = h->cur, odd0 = h->aa_odd;
     cudaGraph_t graph = nullptr;
     HLBM_CUDA(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    int rc = HLBM_OK;
-    for (int k = 0; k < kGraphSteps && rc == HLBM_OK; ++k) rc = step_once(h, h->cap_stream);
+    const int rc = body(h->cap_stream);
     cudaError_t e = cudaStreamEndCapture(h->cap_stream, &graph);
     h->cur = cur0;
     h->aa_odd = odd0;
@@ -177,15 +191,40 @@ int build_graph(hlbm_t* h) {
         return rc;
     }
     if (e != cudaSuccess) return cuda_fail(e);
-    if (h->gexec) {
-        cudaGraphExecDestroy(h->gexec);
-        h->gexec = nullptr;
+    if (*exec) {
+        cudaGraphExecDestroy(*exec);
+        *exec = nullptr;
     }
-    e = cudaGraphInstantiate(&h->gexec, graph, 0);
+    e = cudaGraphInstantiate(exec, graph, 0);
     cudaGraphDestroy(graph);
-    if (e != cudaSuccess) return cuda_fail(e);
-    h->graph_dirty = false;
-    return HLBM_OK;
+    return e == cudaSuccess ? HLBM_OK : cuda_fail(e);
+}
+
+// kGraphSteps steps.
+int build_graph(hlbm_t* h) {
+    const int rc = capture(h, &h->gexec, [h](cudaStream_t s) {
+        int r = HLBM_OK;
+        for (int k = 0; k < kGraphSteps && r == HLBM_OK; ++k) r = step_once(h, s);
+        return r;
+    });
+    if (rc == HLBM_OK) h->graph_dirty = false;
+    return rc;
+}
+
+// kSeriesSamples times `every` steps and the diagnostics, into the records behind out8.
+int build_series(hlbm_t* h, int every) {
+    const int rc = capture(h, &h->series_exec, [h, every](cudaStream_t s) {
+        int r = HLBM_OK;
+        for (int k = 0; k < kSeriesSamples && r == HLBM_OK; ++k) {
+            for (int j = 0; j < every && r == HLBM_OK; ++j) r = step_once(h, s);
+            if (r != HLBM_OK) break;
+            const cudaError_t e = launch_reduce(h->ctx(s), h->layout(), h->state(), h->u_prev, 0, h->partials, h->out8 + 8 * (k + 1));
+            if (e != cudaSuccess) r = cuda_fail(e);
+        }
+        return r;
+    });
+    if (rc == HLBM_OK) h->series_every = every;
+    return rc;
 }
 
 int reset_counters(hlbm_t* h) {
@@ -287,7 +326,7 @@ int hlbm_create(hlbm_t** out, int velset, int nx, int ny, int nz, int storage, i
     if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->varpi, cells * sizeof(float));
     if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->u_prev, 3 * cells * h->arith_bytes());
     if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->partials, nparts * 8 * sizeof(double));
-    if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->out8, 8 * sizeof(double));
+    if (e == cudaSuccess) e = lattice_alloc(h, (void**)&h->out8, (1 + kSeriesSamples) * 8 * sizeof(double));
     if (e == cudaSuccess && !(h->out8_host = slot_acquire())) e = cudaErrorMemoryAllocation;
     if (e == cudaSuccess) e = launch_fill_f32(h->varpi, cells, 1.0f, h->stream);
     if (e != cudaSuccess) {
@@ -338,7 +377,7 @@ int hlbm_set_stream(hlbm_t* h, void* cuda_stream) {
 int hlbm_set_relaxation(hlbm_t* h, double tau) {
     if (!h || !is_finite(tau) || !(tau > 0.5)) return HLBM_ERR_INVALID_ARG;
     h->tau = tau;
-    h->graph_dirty = true;
+    h->settings_changed();
     return HLBM_OK;
 }
 
@@ -347,7 +386,7 @@ int hlbm_set_force(hlbm_t* h, double Fx, double Fy, double Fz) {
     h->F[0] = Fx;
     h->F[1] = Fy;
     h->F[2] = h->q == HLBM_D2Q9 ? 0.0 : Fz;
-    h->graph_dirty = true;
+    h->settings_changed();
     return HLBM_OK;
 }
 
@@ -370,7 +409,7 @@ int hlbm_set_boundary(hlbm_t* h, int axis, int type) {
         if (e != cudaSuccess) return cuda_fail(e);
     }
     h->bc[axis] = type;
-    h->graph_dirty = true;
+    h->settings_changed();
     return HLBM_OK;
 }
 
@@ -378,14 +417,14 @@ int hlbm_set_homogenization(hlbm_t* h, int form) {
     if (!h || (form != HLBM_HOMOG_SHIFT && form != HLBM_HOMOG_DRAG)) return HLBM_ERR_INVALID_ARG;
     if (form == HLBM_HOMOG_DRAG && h->aniso) return HLBM_ERR_STATE;  // the tensor form is a shift form
     h->homog = form;
-    h->graph_dirty = true;
+    h->settings_changed();
     return HLBM_OK;
 }
 
 int hlbm_set_step_kernel(hlbm_t* h, int variant) {
     if (!h || (variant != HLBM_STEP_AUTO && variant != HLBM_STEP_PER_CELL)) return HLBM_ERR_INVALID_ARG;
     h->step_variant = variant;
-    h->graph_dirty = true;
+    h->settings_changed();
     return HLBM_OK;
 }
 
@@ -396,7 +435,7 @@ int hlbm_set_storage_scale(hlbm_t* h, double s) {
     const double m = std::frexp(s, &ex);
     if (m != 0.5 || s < 1.0 || s > 1048576.0) return HLBM_ERR_INVALID_ARG;
     h->scale = s;
-    h->graph_dirty = true;
+    h->settings_changed();
     return HLBM_OK;
 }
 
@@ -419,7 +458,7 @@ int hlbm_porosity_from_permeability(const float* K, double nu, double tau, float
 static void use_scalar_porosity(hlbm_t* h) {
     if (h->aniso) {
         h->aniso = 0;
-        h->graph_dirty = true;
+        h->settings_changed();
     }
 }
 
@@ -475,7 +514,7 @@ int hlbm_set_solid_mask(hlbm_t* h, const unsigned char* solid, int on_device) {
             cudaFree(h->links);
             h->links = nullptr;
         }
-        h->graph_dirty = true;
+        h->settings_changed();
         return HLBM_OK;
     }
     // the state's layout (AA) depends on the obstacles: keep the post-collision
@@ -493,7 +532,7 @@ int hlbm_set_solid_mask(hlbm_t* h, const unsigned char* solid, int on_device) {
     cudaFreeAsync(tmp, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(e);
-    h->graph_dirty = true;
+    h->settings_changed();
     return HLBM_OK;
 }
 
@@ -521,7 +560,7 @@ int hlbm_set_porosity_tensor(hlbm_t* h, const float* varpi3, int on_device) {
         HLBM_CUDA(cudaMemcpyAsync(h->varpi3, varpi3, n * sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
     }
     h->aniso = 1;
-    h->graph_dirty = true;
+    h->settings_changed();
     return HLBM_OK;
 }
 
@@ -669,13 +708,32 @@ int hlbm_reduce_series(hlbm_t* h, long nsamples, int every, double* out, int on_
     double* dst = out;
     if (!on_device) HLBM_CUDA(scratch_alloc(h, (void**)&dst, bytes));
     int rc = HLBM_OK;
-    for (long k = 0; k < nsamples && rc == HLBM_OK; ++k) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    bool graphs = every < kResidentMin && nsamples >= kSeriesMin;
+    if (graphs && (cudaStreamIsCapturing(h->stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone)) {
+        (void)cudaGetLastError();
+        graphs = false;  // a caller's capture takes the single launches
+    }
+    for (long k = 0; k < nsamples && rc == HLBM_OK;) {
+        if (graphs && k && nsamples - k >= kSeriesSamples && at_graph_origin(h)) {
+            if (h->series_every != every) rc = build_series(h, every);
+            if (rc != HLBM_OK) break;
+            cudaError_t e = cudaGraphLaunch(h->series_exec, h->stream);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(dst + 8 * k, h->out8 + 8, kSeriesSamples * 8 * sizeof(double), cudaMemcpyDeviceToDevice,
+                                    h->stream);
+            if (e != cudaSuccess) rc = cuda_fail(e);
+            h->step += (long long)kSeriesSamples * every;
+            k += kSeriesSamples;
+            continue;
+        }
         if (k) rc = hlbm_step(h, every);
         if (rc == HLBM_OK) {
             const cudaError_t e = launch_reduce(h->ctx(h->stream), h->layout(), h->state(), h->u_prev, 0,
                                                 h->partials, dst + 8 * k);
             if (e != cudaSuccess) rc = cuda_fail(e);
         }
+        ++k;
     }
     if (!on_device) {
         cudaError_t e = cudaSuccess;
@@ -860,7 +918,7 @@ int hlbm_load(hlbm_t* h, const char* path) {
     }
     h->scale = hd.scale;
     h->homog = hd.pad == HLBM_HOMOG_DRAG ? HLBM_HOMOG_DRAG : HLBM_HOMOG_SHIFT;
-    h->graph_dirty = true;
+    h->settings_changed();
     HLBM_CUDA(cudaMemcpyAsync(h->buf[0], st.data(), st.size(), cudaMemcpyHostToDevice, h->stream));
     HLBM_CUDA(cudaMemcpyAsync(h->varpi, vp.data(), vp.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream));
     HLBM_CUDA(cudaMemsetAsync(h->u_prev, 0, 3 * h->cells * h->arith_bytes(), h->stream));
