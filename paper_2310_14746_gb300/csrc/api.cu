@@ -172,6 +172,20 @@ int step_once(hlbm_t* h, cudaStream_t s) {
     return HLBM_OK;
 }
 
+bool two_steps(const hlbm_t* h) { return h->pattern == HLBM_TWO_LATTICE && step2_applies(h->ctx(h->stream)); }
+
+// n steps on `s`, where `two` in pairs of two-step launches: four steps then end in the buffer
+// that they began in, as single steps do (a caller may capture them and replay the graph).
+int steps_on(hlbm_t* h, cudaStream_t s, long n, bool two) {
+    int rc = HLBM_OK;
+    for (; two && n >= 4; n -= 4) {
+        HLBM_CUDA(launch_step2(h->ctx(s), h->buf[h->cur], h->buf[1 - h->cur], h->varpi));
+        HLBM_CUDA(launch_step2(h->ctx(s), h->buf[1 - h->cur], h->buf[h->cur], h->varpi));
+    }
+    for (; n > 0 && rc == HLBM_OK; --n) rc = step_once(h, s);
+    return rc;
+}
+
 bool at_graph_origin(const hlbm_t* h) { return h->pattern == HLBM_TWO_LATTICE ? h->cur == 0 : h->aa_odd == 0; }
 
 // Capture what `body` launches on the handle's capture stream, starting from the graph origin layout,
@@ -202,11 +216,8 @@ int capture(hlbm_t* h, cudaGraphExec_t* exec, Body&& body) {
 
 // kGraphSteps steps.
 int build_graph(hlbm_t* h) {
-    const int rc = capture(h, &h->gexec, [h](cudaStream_t s) {
-        int r = HLBM_OK;
-        for (int k = 0; k < kGraphSteps && r == HLBM_OK; ++k) r = step_once(h, s);
-        return r;
-    });
+    const bool two = two_steps(h);
+    const int rc = capture(h, &h->gexec, [h, two](cudaStream_t s) { return steps_on(h, s, kGraphSteps, two); });
     if (rc == HLBM_OK) h->graph_dirty = false;
     return rc;
 }
@@ -627,6 +638,7 @@ int hlbm_step(hlbm_t* h, long nsteps) {
             h->step += n;
         }
     }
+    const bool two = left >= 4 && two_steps(h);
     while (left > 0) {
         if (left >= kGraphSteps && at_graph_origin(h)) {
             if (h->graph_dirty || !h->gexec) {
@@ -637,10 +649,11 @@ int hlbm_step(hlbm_t* h, long nsteps) {
             left -= kGraphSteps;
             h->step += kGraphSteps;
         } else {
-            int rc = step_once(h, h->stream);
+            const int n = two && left >= 4 && left < kGraphSteps ? 4 : 1;
+            int rc = steps_on(h, h->stream, n, two);
             if (rc != HLBM_OK) return rc;
-            --left;
-            ++h->step;
+            left -= n;
+            h->step += n;
         }
     }
     return HLBM_OK;

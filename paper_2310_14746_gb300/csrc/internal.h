@@ -52,6 +52,9 @@ cudaError_t launch_build_links(const LaunchCtx& c, const unsigned char* solid, u
 // (== fin for the AA modes).
 cudaError_t launch_step(const LaunchCtx& c, int mode, const void* fin, void* fout,
                         const float* varpi);
+// Two steps of a two-lattice state in one launch (k_step2.cu), where step2_applies.
+bool step2_applies(const LaunchCtx& c);
+cudaError_t launch_step2(const LaunchCtx& c, const void* fin, void* fout, const float* varpi);
 
 // Many time steps of a small two-lattice state in one launch, in place on `f`
 // (NATURAL layout), with the state resident in the shared memory of one
