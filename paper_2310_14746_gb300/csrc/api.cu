@@ -35,8 +35,9 @@ constexpr int kGraphSteps = 8;  // even: a graph returns the state to its starti
 constexpr long kResidentMin = 6, kResidentMax = 1000;
 // Samples of hlbm_reduce_series per graph replay. Even, so that a replay returns the state to its
 // starting layout. Launched one by one, the three kernels of a sample leave the GPU idle for about
-// a third of a 64^3 sample (step 5.5, diagnostics 9 us). A series of 200 samples, us: 24^3
-// 3290 -> 2210, 48^3 3700 -> 2670, 64^3 4400 -> 3180, 128^3 21260 -> 19980.
+// a third of a 64^3 sample (step 5.5, diagnostics 9 us). A series of 200 samples, us, launched /
+// replayed / replayed with the diagnostics on a branch: 24^3 3290 / 2210 / 1970, 48^3 3700 /
+// 2670 / 2170, 64^3 4360 / 3180 / 2490, 96^3 10180 / 8850 / 7360, 128^3 21270 / 19980 / 18330.
 constexpr int kSeriesSamples = 8;
 constexpr long kSeriesMin = 32;  // shorter series do not pay for the capture
 
@@ -72,6 +73,8 @@ struct hlbm_lattice {
     bool graph_dirty = true;
     cudaGraphExec_t series_exec = nullptr;  // kSeriesSamples samples of hlbm_reduce_series
     int series_every = 0;                   // steps between its samples; 0: to be captured again
+    cudaStream_t series_stream = nullptr;   // capture stream of its diagnostics
+    cudaEvent_t series_ev[3] = {};
     void settings_changed() {
         graph_dirty = true;
         series_every = 0;
@@ -148,6 +151,9 @@ cudaError_t lattice_alloc(hlbm_t* h, void** p, size_t bytes) {
 void free_all(hlbm_t* h) {
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     if (h->series_exec) cudaGraphExecDestroy(h->series_exec);
+    for (cudaEvent_t e : h->series_ev)
+        if (e) cudaEventDestroy(e);
+    if (h->series_stream) cudaStreamDestroy(h->series_stream);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     void* const blocks[] = {h->buf[0], h->buf[1], h->varpi, h->u_prev, h->partials, h->out8};
     for (void* p : blocks)
@@ -222,17 +228,35 @@ int build_graph(hlbm_t* h) {
     return rc;
 }
 
-// kSeriesSamples times `every` steps and the diagnostics, into the records behind out8.
+// kSeriesSamples times `every` steps and the diagnostics, into the records behind out8. The
+// diagnostics of a sample run beside the steps that follow it, up to the one that overwrites
+// the state they read (in place, that is the next one).
 int build_series(hlbm_t* h, int every) {
+    if (!h->series_stream) HLBM_CUDA(cudaStreamCreateWithFlags(&h->series_stream, cudaStreamNonBlocking));
+    for (cudaEvent_t& e : h->series_ev)
+        if (!e) HLBM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     const int rc = capture(h, &h->series_exec, [h, every](cudaStream_t s) {
-        int r = HLBM_OK;
-        for (int k = 0; k < kSeriesSamples && r == HLBM_OK; ++k) {
-            for (int j = 0; j < every && r == HLBM_OK; ++j) r = step_once(h, s);
-            if (r != HLBM_OK) break;
-            const cudaError_t e = launch_reduce(h->ctx(s), h->layout(), h->state(), h->u_prev, 0, h->partials, h->out8 + 8 * (k + 1));
-            if (e != cudaSuccess) r = cuda_fail(e);
+        const bool in_place = h->pattern != HLBM_TWO_LATTICE;
+        cudaStream_t d = h->series_stream;
+        bool read[2] = {};  // by diagnostics that the steps have not waited for
+        for (int k = 0; k < kSeriesSamples; ++k) {
+            for (int j = 0; j < every; ++j) {
+                const int to = in_place ? 0 : 1 - h->cur;
+                if (read[to]) HLBM_CUDA(cudaStreamWaitEvent(s, h->series_ev[to], 0));
+                read[to] = false;
+                const int r = step_once(h, s);
+                if (r != HLBM_OK) return r;
+            }
+            HLBM_CUDA(cudaEventRecord(h->series_ev[2], s));
+            HLBM_CUDA(cudaStreamWaitEvent(d, h->series_ev[2], 0));
+            HLBM_CUDA(launch_reduce(h->ctx(d), h->layout(), h->state(), h->u_prev, 0, h->partials, h->out8 + 8 * (k + 1)));
+            const int from = in_place ? 0 : h->cur;
+            HLBM_CUDA(cudaEventRecord(h->series_ev[from], d));
+            read[from] = true;
         }
-        return r;
+        for (int b = 0; b < 2; ++b)
+            if (read[b]) HLBM_CUDA(cudaStreamWaitEvent(s, h->series_ev[b], 0));
+        return (int)HLBM_OK;
     });
     if (rc == HLBM_OK) h->series_every = every;
     return rc;
