@@ -28,7 +28,10 @@ int cuda_fail(cudaError_t e) {
         if (e_ != cudaSuccess) return cuda_fail(e_);  \
     } while (0)
 
-constexpr int kGraphSteps = 8;  // even: a graph returns the state to its starting layout
+// Steps of the two step graphs: the long one while a run has as many left, the short one below.
+// Even: a graph returns the state to its starting layout. A replay costs about 3 us beside its kernels
+// (kernels chained, us per step, 8 / 16 / 32 / 64 steps: 32^3 2.31 / 2.05 / 2.01 / 1.95).
+constexpr int kGraphSteps[] = {8, 16};
 // Runs of a small lattice that one resident launch takes: below kResidentMin the launch and its
 // loads and stores (about 5 us) cost more than single steps; kResidentMax bounds one launch to
 // about a millisecond or two.
@@ -69,14 +72,15 @@ struct hlbm_lattice {
     double* partials = nullptr;
     double* out8 = nullptr;
     double* out8_host = nullptr;
-    cudaGraphExec_t gexec = nullptr;
-    bool graph_dirty = true;
+    cudaGraphExec_t gexec[2] = {};  // of kGraphSteps
+    bool graph_valid[2] = {};       // captured with the present settings?
+    bool chaining = false;          // capturing a step graph
     cudaGraphExec_t series_exec = nullptr;  // kSeriesSamples samples of hlbm_reduce_series
     int series_every = 0;                   // steps between its samples; 0: to be captured again
     cudaStream_t series_stream = nullptr;   // capture stream of its diagnostics
     cudaEvent_t series_ev[3] = {};
     void settings_changed() {
-        graph_dirty = true;
+        graph_valid[0] = graph_valid[1] = false;
         series_every = 0;
     }
     int step_variant = HLBM_STEP_AUTO;
@@ -108,6 +112,7 @@ struct hlbm_lattice {
         c.varpi3 = aniso ? varpi3 : nullptr;
         c.links = links;
         c.variant = step_variant;
+        c.chained = chaining;
         return c;
     }
 };
@@ -149,7 +154,8 @@ cudaError_t lattice_alloc(hlbm_t* h, void** p, size_t bytes) {
 }
 
 void free_all(hlbm_t* h) {
-    if (h->gexec) cudaGraphExecDestroy(h->gexec);
+    for (cudaGraphExec_t e : h->gexec)
+        if (e) cudaGraphExecDestroy(e);
     if (h->series_exec) cudaGraphExecDestroy(h->series_exec);
     for (cudaEvent_t e : h->series_ev)
         if (e) cudaEventDestroy(e);
@@ -220,11 +226,14 @@ int capture(hlbm_t* h, cudaGraphExec_t* exec, Body&& body) {
     return e == cudaSuccess ? HLBM_OK : cuda_fail(e);
 }
 
-// kGraphSteps steps.
-int build_graph(hlbm_t* h) {
+// Step graph k. In place (AA) a kernel overwrites what it reads, so its successor must not start
+// early: the caches of an SM may hold values from before the overwriting.
+int build_graph(hlbm_t* h, int k) {
     const bool two = two_steps(h);
-    const int rc = capture(h, &h->gexec, [h, two](cudaStream_t s) { return steps_on(h, s, kGraphSteps, two); });
-    if (rc == HLBM_OK) h->graph_dirty = false;
+    h->chaining = h->pattern == HLBM_TWO_LATTICE;
+    const int rc = capture(h, &h->gexec[k], [h, k, two](cudaStream_t s) { return steps_on(h, s, kGraphSteps[k], two); });
+    h->chaining = false;
+    h->graph_valid[k] = rc == HLBM_OK;
     return rc;
 }
 
@@ -664,16 +673,17 @@ int hlbm_step(hlbm_t* h, long nsteps) {
     }
     const bool two = left >= 4 && two_steps(h);
     while (left > 0) {
-        if (left >= kGraphSteps && at_graph_origin(h)) {
-            if (h->graph_dirty || !h->gexec) {
-                int rc = build_graph(h);
+        if (left >= kGraphSteps[0] && at_graph_origin(h)) {
+            const int k = left >= kGraphSteps[1];
+            if (!h->graph_valid[k]) {
+                int rc = build_graph(h, k);
                 if (rc != HLBM_OK) return rc;
             }
-            HLBM_CUDA(cudaGraphLaunch(h->gexec, h->stream));
-            left -= kGraphSteps;
-            h->step += kGraphSteps;
+            HLBM_CUDA(cudaGraphLaunch(h->gexec[k], h->stream));
+            left -= kGraphSteps[k];
+            h->step += kGraphSteps[k];
         } else {
-            const int n = two && left >= 4 && left < kGraphSteps ? 4 : 1;
+            const int n = two && left >= 4 && left < kGraphSteps[0] ? 4 : 1;
             int rc = steps_on(h, h->stream, n, two);
             if (rc != HLBM_OK) return rc;
             left -= n;

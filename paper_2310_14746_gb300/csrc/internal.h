@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <cstddef>
 #include <cstdint>
+#include <utility>
 
 namespace hlbm {
 
@@ -25,7 +26,37 @@ struct LaunchCtx {
     const float* varpi3 = nullptr; // diagonal porosity tensor [3][cells], or null (isotropic)
     const unsigned* links = nullptr; // solid-link masks (resolved obstacles), or null
     int variant = 0;                 // 0: fastest applicable step kernel; 1: per-cell kernel only
+    bool chained = false;            // the kernel before is a step of the same run (see launch_chained)
 };
+
+#ifdef __CUDACC__
+// Launch of a kernel that begins with chain_wait. Where `chained`, its blocks are placed while the
+// kernel before it on the stream still runs, so that its launch costs no time between the two.
+// Measured, us per step in a graph of 16, plain -> chained: FP32 24^3 2.05 -> 1.69, 32^3 2.43 ->
+// 2.05, 64^3 5.51 -> 5.23, 96^3 20.8 -> 20.3; FP16 32^3 2.56 -> 2.05, 48^3 3.20 -> 2.69; slower
+// where the early blocks unbalance the SMs: 48x52x44 with walls 4.74 -> 4.94.
+template <class... P, class... A>
+cudaError_t launch_chained(bool chained, void (*kern)(P...), dim3 grd, dim3 blk, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grd;
+    cfg.blockDim = blk;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, P(std::forward<A>(args))...);
+}
+// Waits until the kernel before has ended and its stores are visible, then lets the next kernel's
+// blocks be placed: at most two kernels overlap, and every load of the caller happens after the
+// end of the kernel that wrote its operands. `x` takes part in every address, so no load can be
+// moved before the wait.
+__device__ __forceinline__ void chain_wait(int& x) {
+    asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" : "+r"(x) : : "memory");
+}
+#endif
 
 // Block of a one-thread-per-cell kernel: a whole row of x as long as it fits 256
 // threads (at least 128 threads), a longer row in equal pieces where that leaves

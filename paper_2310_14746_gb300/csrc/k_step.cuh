@@ -54,7 +54,8 @@ k_step(Planes<const typename S::T, Q> fin, Planes<typename S::T, Q> fout, const 
        Geometry g, Phys<typename S::C> ph, typename S::C s, typename S::C inv_s, int fx_only, int drag,
        const float* __restrict__ varpi3, const unsigned* __restrict__ links) {
     using C = typename S::C;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
+    chain_wait(x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     if (x >= g.nx || y >= g.ny) return;
@@ -127,21 +128,16 @@ cudaError_t step_impl(const LaunchCtx& c, int mode, const void* fin, void* fout,
     const int fx = (Q == 9 || c.F[2] == 0.0) && c.F[1] == 0.0;
     switch (mode) {
         case MODE_TWO_LATTICE:
-            k_step<Q, S, WALLS, MODE_TWO_LATTICE, I, FORM><<<grd, blk, 0, c.stream>>>(a, b, varpi, g, ph, s, inv_s, fx,
-                                                                                    c.drag, c.varpi3, c.links);
-            break;
+            return launch_chained(c.chained, k_step<Q, S, WALLS, MODE_TWO_LATTICE, I, FORM>, grd, blk, 0, c.stream, a, b, varpi, g, ph, s, inv_s,
+                                  fx, c.drag, c.varpi3, c.links);
         case MODE_AA_EVEN:
-            k_step<Q, S, WALLS, MODE_AA_EVEN, I, FORM><<<grd, blk, 0, c.stream>>>(a, b, varpi, g, ph, s, inv_s, fx,
-                                                                                c.drag, c.varpi3, c.links);
-            break;
+            return launch_chained(c.chained, k_step<Q, S, WALLS, MODE_AA_EVEN, I, FORM>, grd, blk, 0, c.stream, a, b, varpi, g, ph, s, inv_s,
+                                  fx, c.drag, c.varpi3, c.links);
         case MODE_AA_ODD:
-            k_step<Q, S, WALLS, MODE_AA_ODD, I, FORM><<<grd, blk, 0, c.stream>>>(a, b, varpi, g, ph, s, inv_s, fx,
-                                                                               c.drag, c.varpi3, c.links);
-            break;
-        default:
-            return cudaErrorInvalidValue;
+            return launch_chained(c.chained, k_step<Q, S, WALLS, MODE_AA_ODD, I, FORM>, grd, blk, 0, c.stream, a, b, varpi, g, ph, s, inv_s,
+                                  fx, c.drag, c.varpi3, c.links);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 // The form a launch needs for the handle's settings.

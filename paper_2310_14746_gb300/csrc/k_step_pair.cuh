@@ -247,7 +247,8 @@ k_step_pair(Planes<const typename S::T, Q> fin, Planes<typename S::T, Q> fout, c
     using P = Pair16<S>;
     using L = Lat<Q>;
     using T = typename S::T;
-    const int xp = blockIdx.x * blockDim.x + threadIdx.x;  // pair index along x
+    int xp = blockIdx.x * blockDim.x + threadIdx.x;  // pair index along x
+    chain_wait(xp);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     if (2 * xp >= g.nx || y >= g.ny) return;
@@ -324,9 +325,8 @@ cudaError_t step_pair_impl(const LaunchCtx& c, const void* fin, void* fout, cons
         a.p[i] = static_cast<const T*>(fin) + (size_t)ia * g.N;
         b.p[i] = static_cast<T*>(fout) + (size_t)ib * g.N;
     }
-    k_step_pair<Q, S, FORM, MODE><<<grd, blk, 0, c.stream>>>(a, b, varpi, g, ph, float(c.scale),
-                                                             float(1.0 / c.scale), c.varpi3);
-    return cudaGetLastError();
+    return launch_chained(c.chained, k_step_pair<Q, S, FORM, MODE>, grd, blk, 0, c.stream, a, b, varpi, g, ph, float(c.scale),
+                          float(1.0 / c.scale), c.varpi3);
 }
 
 // The paired kernel covers periodic lattices with an even nx (aligned pair
