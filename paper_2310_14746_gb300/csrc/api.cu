@@ -850,7 +850,7 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
     const size_t N = h->cells;
     const long nsnap = nsteps > 0 ? (nsteps - 1) / every + 1 : 1;
     const int nseg = every > 2 ? every : 2;  // slot 0/1 double as forward ping-pong buffers
-    const LaunchCtx c = h->ctx(h->stream);
+    LaunchCtx c = h->ctx(h->stream);
     Scratch sc(h);
     char *snaps = nullptr, *seg = nullptr;
     float *lam_a = nullptr, *lam_b = nullptr, *gacc = nullptr;
@@ -867,14 +867,22 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
     // forward sweep, keeping f^{k*every}, and in the last segment every state: the reverse sweep
     // starts there, so only the segments before it are recomputed (90 steps kept every 45: 134
     // forward steps instead of 178). The final state goes to slot 0, which no segment uses.
+    // Where nothing needs the state in between, two steps go in one launch, and all kernels are
+    // chained (180 steps of 128^3 kept every 45: 30.4 -> 28.8 ms for the gradient).
     const long last0 = (nsnap - 1) * every;
+    const bool two = step2_applies(c);
+    c.chained = true;
     void* a = snaps;
-    for (long s = 0; s < nsteps; ++s) {
-        const bool keep = (s + 1) % every == 0 && (s + 1) / every < nsnap;
-        const long slot = s + 1 == nsteps ? 0 : (s >= last0 ? s + 1 - last0 : (s + 1) & 1);
-        void* b = keep ? (void*)(snaps + sb * ((s + 1) / every)) : (void*)(seg + sb * slot);
-        HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, a, b, h->varpi));
+    for (long s = 0, flip = 0; s < nsteps;) {
+        const bool pair = two && s + 1 < last0 && (s + 1) % every != 0;
+        const long n = s + (pair ? 2 : 1);  // the state that this launch produces
+        const bool keep = n % every == 0 && n / every < nsnap;
+        const long slot = n == nsteps ? 0 : (n > last0 ? n - last0 : (flip ^= 1));
+        void* b = keep ? (void*)(snaps + sb * (n / every)) : (void*)(seg + sb * slot);
+        if (pair) HLBM_CUDA(launch_step2(c, a, b, h->varpi));
+        else HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, a, b, h->varpi));
         a = b;
+        s = n;
     }
     HLBM_CUDA(launch_plane_flux(c, kNatural, a, plane_x, jdev));
     rc = adopt_natural(h, a, sc);

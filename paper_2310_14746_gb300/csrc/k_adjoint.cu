@@ -33,7 +33,8 @@ k_adjoint_step(const typename S::T* __restrict__ fn, const float* __restrict__ l
                typename S::C inv_s) {
     using C = typename S::C;
     using L = Lat<Q>;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
+    chain_wait(x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     if (x >= g.nx || y >= g.ny) return;
@@ -111,7 +112,7 @@ k_adjoint_step(const typename S::T* __restrict__ fn, const float* __restrict__ l
     // u = (j + F/2)/rho: du/dj = I/rho, du/drho = -u/rho
     const C a_rho = brho - (bux * ux + buy * uy + buz * uz) * inv_rho;
     const C ajx = bux * inv_rho, ajy = buy * inv_rho, ajz = buz * inv_rho;
-    grad[cell] += float(dvp);
+    grad[cell] = __ldcg(grad + cell) + float(dvp);  // from L2: the launch before may still hold the line when this one starts
 
     const C keep = C(1) - omega;
 #pragma unroll
@@ -194,12 +195,10 @@ static cudaError_t adjoint_impl(const LaunchCtx& c, const void* fn, const float*
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     const auto* f = static_cast<const typename S::T*>(fn);
     if ((size_t)Q * g.N < ((size_t)1 << 31))
-        k_adjoint_step<Q, S, WALLS, int><<<grd, blk, 0, c.stream>>>(f, lam_in, lam_out, varpi, grad, g, ph,
-                                                                    C(1.0 / c.scale));
-    else
-        k_adjoint_step<Q, S, WALLS, long long><<<grd, blk, 0, c.stream>>>(f, lam_in, lam_out, varpi, grad, g, ph,
-                                                                          C(1.0 / c.scale));
-    return cudaGetLastError();
+        return launch_chained(c.chained, k_adjoint_step<Q, S, WALLS, int>, grd, blk, 0, c.stream, f, lam_in, lam_out, varpi,
+                              grad, g, ph, C(1.0 / c.scale));
+    return launch_chained(c.chained, k_adjoint_step<Q, S, WALLS, long long>, grd, blk, 0, c.stream, f, lam_in, lam_out,
+                          varpi, grad, g, ph, C(1.0 / c.scale));
 }
 
 template <int Q, class S, class Fn>
