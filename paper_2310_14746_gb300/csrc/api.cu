@@ -230,8 +230,12 @@ int capture(hlbm_t* h, cudaGraphExec_t* exec, Body&& body) {
 // early: the caches of an SM may hold values from before the overwriting.
 int build_graph(hlbm_t* h, int k) {
     const bool two = two_steps(h);
-    h->chaining = h->pattern == HLBM_TWO_LATTICE;
-    const int rc = capture(h, &h->gexec[k], [h, k, two](cudaStream_t s) { return steps_on(h, s, kGraphSteps[k], two); });
+    const int rc = capture(h, &h->gexec[k], [h, k, two](cudaStream_t s) {
+        if (two) return steps_on(h, s, kGraphSteps[k], true);
+        const int r = step_once(h, s);  // launched plainly: it follows whatever came before the graph
+        h->chaining = h->pattern == HLBM_TWO_LATTICE;
+        return r == HLBM_OK ? steps_on(h, s, kGraphSteps[k] - 1, false) : r;
+    });
     h->chaining = false;
     h->graph_valid[k] = rc == HLBM_OK;
     return rc;
@@ -871,7 +875,6 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
     // chained (180 steps of 128^3 kept every 45: 30.4 -> 28.8 ms for the gradient).
     const long last0 = (nsnap - 1) * every;
     const bool two = step2_applies(c);
-    c.chained = true;
     void* a = snaps;
     for (long s = 0, flip = 0; s < nsteps;) {
         const bool pair = two && s + 1 < last0 && (s + 1) % every != 0;
@@ -883,7 +886,9 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
         else HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, a, b, h->varpi));
         a = b;
         s = n;
+        c.chained = true;
     }
+    c.chained = false;
     HLBM_CUDA(launch_plane_flux(c, kNatural, a, plane_x, jdev));
     rc = adopt_natural(h, a, sc);
     if (rc != HLBM_OK) return rc;
@@ -899,6 +904,7 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
             HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, state(k), state(k + 1), h->varpi));
         for (long s = s1 - 1; s >= s0; --s) {
             HLBM_CUDA(launch_adjoint_step(c, state(s - s0), lam_a, lam_b, h->varpi, gacc));
+            c.chained = true;
             float* t = lam_a;
             lam_a = lam_b;
             lam_b = t;

@@ -50,3 +50,21 @@ def test_same_bits_as_single_launches(q, shape, storage, pattern, walls):
         np.testing.assert_array_equal(a.get_populations(), b.get_populations())
     a.close()
     b.close()
+
+
+def test_graph_waits_for_the_work_before_it():
+    """A replay right behind the write of a new state, a copy or another replay starts from that state."""
+    import torch
+    shape = (48, 52, 56)
+    a, b = (_lattice(19, shape, hb.HLBM_F32, hb.HLBM_TWO_LATTICE, False) for _ in range(2))
+    for seed in range(8):
+        f = torch.from_numpy(inputs.random_populations(19, shape, seed=seed, amplitude=0.02)).cuda()
+        for lat in (a, b):
+            hb.hlbm_set_populations(lat.h, f)
+        a.step(16)
+        a.step(24)
+        for _ in range(40):
+            b.step(1)
+        np.testing.assert_array_equal(a.get_populations(), b.get_populations())
+    a.close()
+    b.close()
