@@ -234,7 +234,8 @@ k_batched_step(const DevTable* __restrict__ tab, int k) {
     constexpr int kWords = (int)(sizeof(DevSlot) / sizeof(int));
     constexpr int cls = 2 * S::kind + (FAST ? 1 : 0);
     constexpr bool k16 = S::kind == HLBM_F16DEV || S::kind == HLBM_BF16DEV;
-    const int t = tab->lo[cls] + blockIdx.x;
+    int t = tab->lo[cls] + blockIdx.x;
+    chain_wait(t);
     if (t >= tab->hi[cls]) return;  // uniform over the block
     if ((int)threadIdx.x < kWords)
         reinterpret_cast<int*>(&sl)[threadIdx.x] =
@@ -630,7 +631,8 @@ cudaError_t widen_to_fp32(hlbm_server_t* s, Live& l) {
 // the tile-kernel classes (per step: the reduced-precision classes, then the
 // FP32 ones) on one branch, each large slot's single-lattice launches on one of
 // the other branches (round robin), all forked from and joined into the
-// capture stream.
+// capture stream. The kernels of a branch are chained (12 FP16 requests of up to 96^3
+// 31.3 -> 30.3 ms).
 int build_graph(hlbm_server_t* s) {
     if (!s->cap_stream) SRV_CUDA(cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking));
     if (!s->fork_ev) SRV_CUDA(cudaEventCreateWithFlags(&s->fork_ev, cudaEventDisableTiming));
@@ -656,11 +658,11 @@ int build_graph(hlbm_server_t* s) {
     SRV_CUDA(cudaStreamBeginCapture(s->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaEventRecord(s->fork_ev, s->cap_stream);
     for (int b = 0; b < used && le == cudaSuccess; ++b) le = cudaStreamWaitEvent(s->branch[b], s->fork_ev, 0);
+    bool follows[kGraphBranches] = {};  // the first kernel of a branch is launched plainly (launch_chained)
     const auto launch = [&](auto kern, int blocks, int k) {
-        if (blocks > 0 && le == cudaSuccess) {
-            kern<<<blocks, kBlock, 0, s->branch[0]>>>(s->dtab, k);
-            le = cudaGetLastError();
-        }
+        if (blocks <= 0 || le != cudaSuccess) return;
+        le = launch_chained(follows[0], kern, dim3(blocks), dim3(kBlock), 0, s->branch[0], s->dtab, k);
+        follows[0] = true;
     };
     for (int k = 0; k < s->check_every && le == cudaSuccess; ++k) {
         const int* g = s->grid;
@@ -668,7 +670,10 @@ int build_graph(hlbm_server_t* s) {
             if (le != cudaSuccess) break;
             const Live* l = direct[d];
             LaunchCtx c = s->ctx_for(*l);
-            c.stream = s->branch[first_direct + (int)(d % direct_branches)];
+            const int b = first_direct + (int)(d % direct_branches);
+            c.stream = s->branch[b];
+            c.chained = follows[b];
+            follows[b] = true;
             le = launch_step(c, MODE_TWO_LATTICE, l->ds.f[k & 1], l->ds.f[(k + 1) & 1], l->ds.varpi);
         }
         launch(k_batched_step<StoreF16, true>, g[2 * HLBM_F16DEV + 1], k);
