@@ -3,8 +3,8 @@
 //
 // A single step is bound by HBM: it reads and writes the whole state. This kernel
 // reads the state of step n and writes the state of step n + 2; the state of
-// step n + 1 lives in shared memory only. A block owns an output tile of kTX x kTY
-// cells in (x, y) and marches along z. For every plane p it
+// step n + 1 lives in shared memory only. A block owns an output tile of 32 x 7 or
+// 24 x 9 cells in (x, y) and marches along z. For every plane p it
 //  1. copies the rows that plane p pulls from into a staging buffer (16-byte
 //     asynchronous copies, one plane ahead), pulls and collides the n + 1 populations
 //     of the tile and a halo of one cell (phase 1), and
@@ -24,16 +24,19 @@
 // The collision is the function of the single-step kernels, so two steps here and
 // two single steps give the same bits.
 //
-// What bounds it: no longer HBM alone. Two steps of 256^3 move 2.6 GB (0.40 ms at the copy
-// rate) and take 0.62 ms: the copies, the collisions and the shared-memory traffic of a
-// block's planes add up more than they overlap, and tile halos cost 1.36 times the cells of
-// phase 1. With parts switched off at 192^3 (us per step, complete 136): no copies 103, no
-// stores 115, collisions passed through 124, none of the three 49. Measured against the
-// single-step kernel, us per step: 256^3 373 -> 309, 192^3 160 -> 137, 288^3 533 -> 432,
-// 128^3 49.5 -> 44.2, 160^3 94.8 -> 88.2; single steps run at 1.02 of the copy rate.
+// What bounds it: no longer HBM alone. Two steps of 256^3 move 2.68 GB (0.40 ms at the copy
+// rate) and take 0.62 ms: shared memory allows 15 warps per SM, whose copies, collisions and
+// shared-memory accesses add up more than they overlap (DRAM 51 %, shared memory 41 % busy), and
+// phase 1 works on 1.32 to 1.37 times the cells. With parts switched off at 192^3 (us per step,
+// complete 136): no copies 103, no stores 115, collisions passed through 124, none of the three
+// 49. Measured against the single-step kernel, us per step: 256^3 373 -> 309, 192^3 160 -> 137,
+// 288^3 533 -> 420, 240^3 309 -> 250, 128^3 49.5 -> 44.2, 160^3 94.8 -> 83.6; single steps run at
+// 1.02 of the copy rate.
 // Variants that were slower at 256^3: two larger blocks per SM with the whole
 // window in registers 340, one tensor-map box per direction 341, a bulk copy per row 386,
 // delay lines in registers 337, and every 16-bit variant (bound by instructions).
+#include <cmath>
+
 #include "k_step_pair.cuh"
 
 namespace hlbm {
@@ -42,7 +45,6 @@ namespace {
 
 using L = Lat<19>;
 
-constexpr int kTX = 32, kTY = 7;  // output tile of a block
 constexpr int kBlocksPerSM = 3;
 
 // Position of direction i within the directions of the same c_z, in index order, and
@@ -65,16 +67,20 @@ struct StagedDirs {
 };
 __constant__ const StagedDirs kStaged;
 
-constexpr int EX = kTX + 2, EY = kTY + 2;  // tile with its halo
-constexpr int PX = EX / 2;                 // pairs per extended row
-constexpr int kPairs = PX * EY;
-constexpr int kThreads = (kPairs + 31) / 32 * 32;
-constexpr int PS = EX * EY;  // values of one direction of one n + 1 plane
-constexpr int C = 4;         // floats per 16-byte chunk
-constexpr int kChunks = kTX / C + 2, SX = kChunks * C;  // staged columns x0 - C .. x0 + TX + C - 1
-constexpr int kStage = 19 * SX * EY, kUp = 15 * PS, kFlat = 18 * PS, kDown = 5 * PS;  // floats
-constexpr int kBytes = (kStage + kUp + kFlat + kDown) * (int)sizeof(float);
-static_assert(kBlocksPerSM * (kBytes + 1024) <= 228 * 1024, "blocks per SM");
+// Output tile of TX x TY columns.
+template <int TX, int TY>
+struct Tile {
+    static constexpr int EX = TX + 2, EY = TY + 2;  // with its halo
+    static constexpr int PX = EX / 2;               // pairs per extended row
+    static constexpr int kPairs = PX * EY;
+    static constexpr int kThreads = (kPairs + 31) / 32 * 32;
+    static constexpr int PS = EX * EY;  // values of one direction of one n + 1 plane
+    static constexpr int C = 4;         // floats per 16-byte chunk
+    static constexpr int kChunks = TX / C + 2, SX = kChunks * C;  // staged columns x0 - C .. x0 + TX + C - 1
+    static constexpr int kStage = 19 * SX * EY, kUp = 15 * PS, kFlat = 18 * PS, kDown = 5 * PS;  // floats
+    static constexpr int kBytes = (kStage + kUp + kFlat + kDown) * (int)sizeof(float);
+    static_assert(TX % C == 0 && kChunks <= 32 && kBlocksPerSM * (kBytes + 1024) <= 228 * 1024, "tile");
+};
 
 struct Pops {
     F2 v[19];
@@ -108,30 +114,33 @@ __device__ __forceinline__ void copy16(unsigned dst, const void* src) {
 __device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
 // zc: output planes per block. varpi: [cells], or [3][cells] for the tensor form.
-template <int FORM>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSM)
+template <int FORM, int TX, int TY>
+__global__ void __launch_bounds__(Tile<TX, TY>::kThreads, kBlocksPerSM)
 k_step2(const float* __restrict__ fin, float* __restrict__ fout, const float* __restrict__ varpi, Geometry g,
         Phys<float> ph, int zc) {
+    using K = Tile<TX, TY>;
+    constexpr int EX = K::EX, EY = K::EY, PX = K::PX, PS = K::PS, C = K::C, SX = K::SX;
+    constexpr int kThreads = K::kThreads, kChunks = K::kChunks;
     extern __shared__ __align__(16) float smem[];
-    float* const up = smem + kStage;
-    float* const flat = up + kUp;
-    float* const down = flat + kFlat;
+    float* const up = smem + K::kStage;
+    float* const flat = up + K::kUp;
+    float* const down = flat + K::kFlat;
     const int N = (int)g.N, plane = g.nx * g.ny;
     const int t = threadIdx.x;
-    const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * kTY, z0 = blockIdx.z * zc;
-    const int xe = min(x0 + kTX, g.nx), ye = min(y0 + kTY, g.ny), z1 = min(z0 + zc, g.nz);
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * zc;
+    const int xe = min(x0 + TX, g.nx), ye = min(y0 + TY, g.ny), z1 = min(z0 + zc, g.nz);
 
     // phase 1: the pair at extended position (2 px, py), cells x0 - 1 + 2 px and the next
     const int py = t / PX, px = t - py * PX;
     const int ya = y0 - 1 + py;
-    const bool on1 = t < kPairs && x0 - 1 + 2 * px <= xe && ya <= ye;
+    const bool on1 = t < K::kPairs && x0 - 1 + 2 * px <= xe && ya <= ye;
     const int row1 = wrap1(ya, g.ny) * g.nx;
     const int a1 = row1 + wrap1(x0 - 1 + 2 * px, g.nx), b1 = row1 + wrap1(x0 + 2 * px, g.nx);
     const int w1 = py * EX + 2 * px;  // where the pair lands in an n + 1 plane
     // phase 2: the pair at output position (2 qx, qy)
-    const int qy = t / (kTX / 2), qx = t - qy * (kTX / 2);
+    const int qy = t / (TX / 2), qx = t - qy * (TX / 2);
     const int xo = x0 + 2 * qx, yo = y0 + qy;
-    const bool on2 = qy < kTY && xo < xe && yo < ye;
+    const bool on2 = qy < TY && xo < xe && yo < ye;
     const int cell2 = yo * g.nx + xo;
     const int w2 = (qy + 1) * EX + 2 * qx + 1;
 
@@ -225,38 +234,55 @@ k_step2(const float* __restrict__ fin, float* __restrict__ fout, const float* __
     }
 }
 
-// Planes per block with the least time, in phases of one plane: a block of zc planes runs
-// zc + 2 planes of phase 1 and zc of phase 2, and starts and ends with a wait.
+// Tile and planes per block with the least time, in phases of one plane of the 32 x 7 tile (about
+// 1.75 us for a phase pair with every SM full): a block of zc planes runs zc + 2 planes of phase 1 and zc of
+// phase 2, and starts and ends with a wait; a plane of the 24 x 9 tile takes 0.945 of that; the
+// blocks of a single wave run in step and take 1.03; a last wave that is partly full saves a fifth of
+// what is missing. Two steps, 32 x 7 / 24 x 9, us: 128^3 88.7 / 94.6, 160^3 177 / 167, 240^3
+// 541 / 501, 256^3 617 / 615, 288^3 864 / 840. Over 60 lattices with two to four measured plans
+// each, the plan chosen here took 0.6 % more than the best of them. Slower: 16 x 14 (256^3 671),
+// and with two blocks per SM 48 x 7 (721) and 32 x 11 (651, though 163 at 160^3).
 struct Step2Plan {
+    bool wide;      // 32 x 7, else 24 x 9
     int zc;
     double useful;  // cells over the cells that the waves' blocks have room for
 };
 Step2Plan step2_plan(const LaunchCtx& c) {
     constexpr int kSlots = kBlocksPerSM * 152;
-    Step2Plan best{c.nz, 0.0};
-    const long long bxy = (long long)((c.nx + kTX - 1) / kTX) * ((c.ny + kTY - 1) / kTY);
-    for (int k = 1; k <= c.nz; ++k) {
-        const int zc = (c.nz + k - 1) / k, bz = (c.nz + zc - 1) / zc;
-        const int waves = (int)((bxy * bz + kSlots - 1) / kSlots);
-        const double useful = 2.0 * c.nx * c.ny * c.nz / (waves * (2.0 * zc + 3.0) * kSlots * kTX * kTY);
-        if (useful > best.useful) best = {zc, useful};
-        if (zc <= 8) break;
+    Step2Plan best{true, c.nz, 0.0};
+    for (const bool wide : {true, false}) {
+        const int tx = wide ? 32 : 24, ty = wide ? 7 : 9;
+        const long long bxy = (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty);
+        for (int k = 1; k <= c.nz; ++k) {
+            const int zc = (c.nz + k - 1) / k, bz = (c.nz + zc - 1) / zc;
+            const double full = (double)(bxy * bz) / kSlots, waves = std::ceil(full);
+            const double turns = waves > 1.0 ? waves - 0.2 * (waves - full) : 1.03;
+            const double time = turns * (2.0 * zc + 3.0) * (wide ? 1.0 : 0.945);
+            const double useful = 2.0 * c.nx * c.ny * c.nz / (time * kSlots * 32 * 7);
+            if (useful > best.useful) best = {wide, zc, useful};
+            if (zc <= 8) break;
+        }
     }
     return best;
 }
 
-template <int FORM>
-cudaError_t step2_impl(const LaunchCtx& c, const void* fin, void* fout, const float* varpi) {
-    const auto kern = k_step2<FORM>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+template <int FORM, int TX, int TY>
+cudaError_t step2_tile(const LaunchCtx& c, int zc, const void* fin, void* fout, const float* varpi) {
+    using K = Tile<TX, TY>;
+    const auto kern = k_step2<FORM, TX, TY>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, K::kBytes);
     if (e != cudaSuccess) return e;
     const Geometry g{c.nx, c.ny, c.nz, 0, 0, 0, (size_t)c.nx * c.ny * c.nz};
-    const Step2Plan p = step2_plan(c);
-    const dim3 grd((c.nx + kTX - 1) / kTX, (c.ny + kTY - 1) / kTY, (c.nz + p.zc - 1) / p.zc);
-    kern<<<grd, kThreads, kBytes, c.stream>>>(static_cast<const float*>(fin), static_cast<float*>(fout),
-                                              FORM == FORM_ANISO ? c.varpi3 : varpi, g, make_phys<float, 19>(c.tau, c.F),
-                                              p.zc);
+    const dim3 grd((c.nx + TX - 1) / TX, (c.ny + TY - 1) / TY, (c.nz + zc - 1) / zc);
+    kern<<<grd, K::kThreads, K::kBytes, c.stream>>>(static_cast<const float*>(fin), static_cast<float*>(fout),
+                                                    FORM == FORM_ANISO ? c.varpi3 : varpi, g,
+                                                    make_phys<float, 19>(c.tau, c.F), zc);
     return cudaGetLastError();
+}
+template <int FORM>
+cudaError_t step2_impl(const LaunchCtx& c, const void* fin, void* fout, const float* varpi) {
+    const Step2Plan p = step2_plan(c);
+    return p.wide ? step2_tile<FORM, 32, 7>(c, p.zc, fin, fout, varpi) : step2_tile<FORM, 24, 9>(c, p.zc, fin, fout, varpi);
 }
 
 }  // namespace
@@ -264,16 +290,16 @@ cudaError_t step2_impl(const LaunchCtx& c, const void* fin, void* fout, const fl
 // Periodic FP32 lattices whose rows are whole 16-byte chunks, with 32-bit indices and axes
 // that one wrap correction covers, and whose two states are well above L2 (228 MB: at
 // 96^3 one step per pass is faster, 21.0 vs 23.0 us). The gain follows step2_plan's `useful`;
-// over 95 lattices of 1.5 to 25 M cells it was 1.02 to 1.26 above these limits (force along x),
-// 1.03 to 1.21 (other forces, drag) and 1.03 to 1.10 (tensor, which loads three porosities),
-// and 0.83 to 1.17 below: 144^3 0.995, 100x180x228 0.96, 36x300x300 0.83.
+// over 60 lattices of 1.2 to 25 M cells it was 1.05 to 1.30 above these limits for a force along
+// x, 1.02 to 1.25 for other forces and drag, 1.03 to 1.17 for the tensor, which loads three
+// porosities; below them 0.97 to 1.11, 0.98 to 1.10 and 0.92 to 1.04.
 bool step2_applies(const LaunchCtx& c) {
     const size_t n = (size_t)c.nx * c.ny * c.nz;
     if (c.variant != 0 || c.q != 19 || c.storage != 1 || c.wall[0] || c.wall[1] || c.wall[2] || c.links || c.nx % 4 != 0 ||
         c.nx < 8 || c.ny < 4 || c.nz < 4 || 19 * n >= ((size_t)1 << 31) || n < 1500000)
         return false;
     const int form = step_form(c, 19);
-    return step2_plan(c).useful >= (form == FORM_SHIFT_FX ? 0.78 : (form == FORM_ANISO ? 0.88 : 0.84));
+    return step2_plan(c).useful >= (form == FORM_SHIFT_FX ? 0.78 : (form == FORM_ANISO ? 0.86 : 0.83));
 }
 
 cudaError_t launch_step2(const LaunchCtx& c, const void* fin, void* fout, const float* varpi) {

@@ -35,10 +35,11 @@ def _lattice(shape, form, variant, stream=None):
     return lat
 
 
-# tiles are 32 x 7: rows that end in a narrow tile, in a full one, in one of 4 cells; y and z remainders
+# tiles are 32 x 7 and 24 x 9: rows that end in a narrow tile, in a full one, in one of 4 cells; y and z remainders
 @pytest.mark.parametrize("form", ["fx", "shift", "drag", "tensor"])
 @pytest.mark.parametrize("shape", [(160, 150, 128), (208, 151, 172), (186, 133, 228), (171, 133, 160), (96, 168, 288),
-                                   (159, 152, 132), (384, 384, 32), (64, 63, 1024), (186, 105, 292)])
+                                   (159, 152, 132), (384, 384, 32), (64, 63, 1024), (186, 105, 292),
+                                   (168, 154, 240), (148, 134, 144)])
 def test_same_bits_as_single_steps(shape, form):
     import torch
     a, b = _lattice(shape, form, hb.HLBM_STEP_AUTO), _lattice(shape, form, hb.HLBM_STEP_PER_CELL)
