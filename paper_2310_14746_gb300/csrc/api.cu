@@ -74,7 +74,7 @@ struct hlbm_lattice {
     double* out8_host = nullptr;
     cudaGraphExec_t gexec[2] = {};  // of kGraphSteps
     bool graph_valid[2] = {};       // captured with the present settings?
-    bool chaining = false;          // capturing a step graph
+    int chaining = CHAIN_NONE;      // of the steps that are launched next
     cudaGraphExec_t series_exec = nullptr;  // kSeriesSamples samples of hlbm_reduce_series
     int series_every = 0;                   // steps between its samples; 0: to be captured again
     cudaStream_t series_stream = nullptr;   // capture stream of its diagnostics
@@ -233,10 +233,10 @@ int build_graph(hlbm_t* h, int k) {
     const int rc = capture(h, &h->gexec[k], [h, k, two](cudaStream_t s) {
         if (two) return steps_on(h, s, kGraphSteps[k], true);
         const int r = step_once(h, s);  // launched plainly: it follows whatever came before the graph
-        h->chaining = h->pattern == HLBM_TWO_LATTICE;
+        if (h->pattern == HLBM_TWO_LATTICE) h->chaining = CHAIN_GRAPH;
         return r == HLBM_OK ? steps_on(h, s, kGraphSteps[k] - 1, false) : r;
     });
-    h->chaining = false;
+    h->chaining = CHAIN_NONE;
     h->graph_valid[k] = rc == HLBM_OK;
     return rc;
 }
@@ -886,9 +886,9 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
         else HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, a, b, h->varpi));
         a = b;
         s = n;
-        c.chained = true;
+        c.chained = CHAIN_STREAM;
     }
-    c.chained = false;
+    c.chained = CHAIN_NONE;
     HLBM_CUDA(launch_plane_flux(c, kNatural, a, plane_x, jdev));
     rc = adopt_natural(h, a, sc);
     if (rc != HLBM_OK) return rc;
@@ -904,7 +904,7 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
             HLBM_CUDA(launch_step(c, MODE_TWO_LATTICE, state(k), state(k + 1), h->varpi));
         for (long s = s1 - 1; s >= s0; --s) {
             HLBM_CUDA(launch_adjoint_step(c, state(s - s0), lam_a, lam_b, h->varpi, gacc));
-            c.chained = true;
+            c.chained = CHAIN_STREAM;
             float* t = lam_a;
             lam_a = lam_b;
             lam_b = t;

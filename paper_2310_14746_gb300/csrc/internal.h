@@ -9,6 +9,7 @@
 
 namespace hlbm {
 
+enum Chain { CHAIN_NONE = 0, CHAIN_GRAPH = 1, CHAIN_STREAM = 2 };  // captured into a graph / launched one by one
 enum StepMode { MODE_TWO_LATTICE = 0, MODE_AA_EVEN = 1, MODE_AA_ODD = 2 };
 
 // Everything a launch needs to know about a lattice, in plain types.
@@ -26,7 +27,7 @@ struct LaunchCtx {
     const float* varpi3 = nullptr; // diagonal porosity tensor [3][cells], or null (isotropic)
     const unsigned* links = nullptr; // solid-link masks (resolved obstacles), or null
     int variant = 0;                 // 0: fastest applicable step kernel; 1: per-cell kernel only
-    bool chained = false;            // the kernel before is a step of the same run (see launch_chained)
+    int chained = CHAIN_NONE;        // is the kernel before one of the same run? (see launch_chained)
 };
 
 #ifdef __CUDACC__
@@ -36,11 +37,22 @@ struct LaunchCtx {
 // kernel of a graph, or one that follows a graph or a copy, is launched plainly (with the attribute
 // such kernels have been seen to start before that work had ended).
 // Measured, us per step in a graph of 16, plain -> chained: FP32 24^3 2.05 -> 1.69, 32^3 2.43 ->
-// 2.05, 64^3 5.51 -> 5.23, 96^3 20.8 -> 20.3; FP16 32^3 2.56 -> 2.05, 48^3 3.20 -> 2.69; slower
-// where the early blocks unbalance the SMs: 48x52x44 with walls 4.74 -> 4.94.
+// 2.05, 64^3 5.51 -> 5.23, 96^3 20.8 -> 20.3; FP16 32^3 2.56 -> 2.05, 48^3 3.20 -> 2.69. Where two
+// grids do not fit the chip together, but one leaves room, the early blocks crowd the SMs that are
+// free first, and the others stay idle: 45^3 (0.68 of the blocks that fit) 3.64 -> 3.99, 41x44x39
+// with walls (0.56) 4.23 -> 5.10, but 36^3 (0.43) 3.07 -> 2.69 and 51^3 (0.87) 4.72 -> 4.36. So grids
+// between 0.44 and 0.78 are launched plainly in a graph (one by one, where the gaps are
+// longer, chained: 48^3 gradient 1.60 against 1.87 ms).
 // Launched one by one, a 48^3 gradient over 90 steps takes 1.60 instead of 2.10 ms.
 template <class... P, class... A>
-cudaError_t launch_chained(bool chained, void (*kern)(P...), dim3 grd, dim3 blk, size_t smem, cudaStream_t s, A&&... args) {
+cudaError_t launch_chained(int chained, void (*kern)(P...), dim3 grd, dim3 blk, size_t smem, cudaStream_t s, A&&... args) {
+    if (chained == CHAIN_GRAPH) {
+        int fit = 0;  // blocks per SM
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, (int)(blk.x * blk.y * blk.z), smem) == cudaSuccess) {
+            const double share = (double)grd.x * grd.y * grd.z / (152.0 * fit);
+            if (share > 0.44 && share < 0.78) chained = CHAIN_NONE;
+        }
+    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grd;
     cfg.blockDim = blk;

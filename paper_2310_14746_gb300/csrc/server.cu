@@ -658,11 +658,11 @@ int build_graph(hlbm_server_t* s) {
     SRV_CUDA(cudaStreamBeginCapture(s->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaEventRecord(s->fork_ev, s->cap_stream);
     for (int b = 0; b < used && le == cudaSuccess; ++b) le = cudaStreamWaitEvent(s->branch[b], s->fork_ev, 0);
-    bool follows[kGraphBranches] = {};  // the first kernel of a branch is launched plainly (launch_chained)
+    int follows[kGraphBranches] = {};  // the first kernel of a branch is launched plainly (launch_chained)
     const auto launch = [&](auto kern, int blocks, int k) {
         if (blocks <= 0 || le != cudaSuccess) return;
         le = launch_chained(follows[0], kern, dim3(blocks), dim3(kBlock), 0, s->branch[0], s->dtab, k);
-        follows[0] = true;
+        follows[0] = CHAIN_GRAPH;
     };
     for (int k = 0; k < s->check_every && le == cudaSuccess; ++k) {
         const int* g = s->grid;
@@ -673,7 +673,7 @@ int build_graph(hlbm_server_t* s) {
             const int b = first_direct + (int)(d % direct_branches);
             c.stream = s->branch[b];
             c.chained = follows[b];
-            follows[b] = true;
+            follows[b] = CHAIN_GRAPH;
             le = launch_step(c, MODE_TWO_LATTICE, l->ds.f[k & 1], l->ds.f[(k + 1) & 1], l->ds.varpi);
         }
         launch(k_batched_step<StoreF16, true>, g[2 * HLBM_F16DEV + 1], k);
