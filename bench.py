@@ -11,8 +11,10 @@ value : MLUPS = cells * time steps / device time (CUDA events, max over ranks).
 e2e   : the same metric through the C ABI with host buffers: per step the porosity field
         is copied from pinned host memory (set_porosity), the lattice re-initialised,
         100 time steps run and the diagnostics read back to the host.
-roofline : the stream-collide kernel's algorithmic bytes (q*2*sizeof(T) + 4 per cell
-        update) over its average launch time, against the measured HBM copy bandwidth.
+roofline : the stream-collide kernel's algorithmic bytes (q*2*sizeof(T) + 4 per cell and
+        launch) over its average launch time, against the measured HBM copy bandwidth. A
+        launch of the FP32 two-lattice workloads advances two steps (steps_per_launch), so
+        its bytes per cell update are half of that.
 cpu_baseline : the FP64 CPU oracle timed on the host cores on a bounded sample (a few
         time steps of the same 256^3 workload).
 
@@ -57,8 +59,8 @@ KERNEL_TRAFFIC_BYTES = {
     # (1342250752 + 1228698112 and 1342237696 + 1217931008 bytes)
     ("stream_collide_d3q19_f32_two", 256): {"bytes": 2565558784, "source_hash": "76d4a47919d1105a"},
     # k_step<19, StoreF32, periodic, AA even / AA odd, int, shift-fx>, 256^3: mean of the even
-    # (1342202368 + 1217577984) and odd (1342190336 + 1217456640 bytes) launch of one capture
-    ("stream_collide_d3q19_f32_aa", 256): {"bytes": 2559713664, "source_hash": "76d4a47919d1105a"},
+    # (1342405120 + 1216537856) and odd (1342217728 + 1214018048 bytes) launch of one capture
+    ("stream_collide_d3q19_f32_aa", 256): {"bytes": 2557589376, "source_hash": "1773fb175a24e720"},
     # k_step_pair<19, StoreF16, shift-fx, two-lattice>, 384^3 Boolean sphere matrix: mean of two launches
     # (2378278656 + 2107357184 and 2378211072 + 2106170112 bytes)
     ("stream_collide_d3q19_f16_two", 384): {"bytes": 4485008512, "source_hash": "59ee95aa12972e25"},
@@ -78,6 +80,12 @@ KERNEL_SOURCES = {
     "f16": _COMMON_SOURCES + ("k_step_pair.cuh", "k_step_f16.cu"),
     "bf16": _COMMON_SOURCES + ("k_step_pair.cuh", "k_step_bf16.cu"),
 }
+
+
+def steps_per_launch(w):
+    """Time steps that one launch of the workload's step kernel advances: two for the periodic FP32
+    two-lattice cubes here, all larger than L2 (csrc/k_step2.cu), else one."""
+    return 2 if w["q"] == 19 and w["storage"] == "f32" and w["pattern"] == "two" else 1
 
 
 def kernel_source_hash(kname):
@@ -431,7 +439,8 @@ def aa_leg(args, w, field, stream):
 def adjoint_leg(n=128, nsteps=2000, every=45, period=32, ratio=0.3, tau=0.6, F=(1e-6, 0.0, 0.0)):
     """Gradient of the outflow flux w.r.t. varpi on the adjoint workload (128^3 regular spheres,
     2000 steps, state kept every 45 steps): wall time of the whole call and its algorithmic
-    bytes (forward run + segment recomputation at 156 B/LUP, reverse steps at 240 B/LUP)."""
+    bytes: 156 per cell and forward launch (two steps each where no state in between is kept, single
+    ones in the last segment and when a segment is recomputed), 240 per cell and reverse step."""
     import torch
     import paper_2310_14746_gb300 as hb
     from paper_2310_14746_gb300 import inputs
@@ -452,7 +461,8 @@ def adjoint_leg(n=128, nsteps=2000, every=45, period=32, ratio=0.3, tau=0.6, F=(
     lat.close()
     cells = n ** 3
     nsnap = (nsteps - 1) // every + 1
-    algo = cells * ((2 * nsteps - nsnap) * 156 + nsteps * 240)
+    forward = (nsnap - 1) * (every // 2 + every % 2) + nsteps - (nsnap - 1) * every
+    algo = cells * ((forward + (nsnap - 1) * (every - 1)) * 156 + nsteps * 240)
     peak, kind = measured_hbm_peak()
     return {"workload": "D3Q19 %d^3 regular spheres (period %d, r = %.1f P), %d steps, checkpoint every %d"
                         % (n, period, ratio, nsteps, every),
@@ -739,7 +749,9 @@ def run_gpu(args, w, rank, world, local_rank):
     lat.set_porosity(varpi_pinned.numpy())
     lat.init_equilibrium()
 
-    launches_per_step = inner + 2  # stream-collide launches + 2 reduction kernels
+    per_launch = steps_per_launch(w)
+    # stream-collide launches (two-step ones in pairs, the last one to three steps single) + 2 reduction kernels
+    launches_per_step = (inner if per_launch == 1 else inner // 4 * 2 + inner % 4) + 2
 
     def one_step(ev_a=None, ev_b=None):
         if ev_a is not None:
@@ -788,7 +800,7 @@ def run_gpu(args, w, rank, world, local_rank):
     h2d = cells * 4 + q * 8
     d2h = 8 * 8
 
-    bytes_per_lup = 2 * q * hb.STORAGE_BYTES[storage] + 4
+    bytes_per_lup = (2 * q * hb.STORAGE_BYTES[storage] + 4) / per_launch
     achieved = bytes_per_lup * cells / (kern_ms * 1e-3) / 1e9
     peak, peak_kind = measured_hbm_peak()
     kname = "stream_collide_d%dq%d_%s_%s" % (3 if q == 19 else 2, q, w["storage"], w["pattern"])
@@ -832,7 +844,8 @@ def run_gpu(args, w, rank, world, local_rank):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic, "traffic_note": traffic_note,
                          "kernel_source_hash": kernel_source_hash(kname), "peak_kind": peak_kind,
-                         "kernel": kname, "kernel_ms": kern_ms, "bytes_per_lup": bytes_per_lup},
+                         "kernel": kname, "kernel_ms": kern_ms * per_launch, "steps_per_launch": per_launch,
+                         "bytes_per_lup": bytes_per_lup},
             "e2e": {"value": e2e_value, "unit": "MLUPS", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
             "gpu_launches": launches_per_step * args.steps,
             "clocks": clk.summary(),

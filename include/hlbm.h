@@ -229,7 +229,7 @@ int hlbm_get_populations(hlbm_t* h, double* f, int on_device);
 /* ---- time stepping ----------------------------------------------------- */
 
 /* Advance nsteps >= 0 time steps (stream + collide, see above). Asynchronous.
- * Runs of at least 8 steps replay a captured CUDA graph of the step
+ * Runs of at least 8 steps replay captured CUDA graphs of the step
  * sequence; shorter runs launch directly. */
 int hlbm_step(hlbm_t* h, long nsteps);
 
