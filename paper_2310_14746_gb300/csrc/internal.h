@@ -146,7 +146,8 @@ size_t storage_bytes(int storage);
 bool pool_keeps(size_t bytes);  // does a released pool keep this much mapped?
 cudaError_t pool_acquire(cudaMemPool_t* pool);
 void pool_release(cudaMemPool_t pool);
-cudaError_t pool_shared(cudaMemPool_t* pool);  // the servers' pool
+// The servers' pool; where nothing is kept, a new one that the caller destroys (own).
+cudaError_t pool_shared(cudaMemPool_t* pool, bool* own);
 cudaError_t pool_alloc(cudaMemPool_t pool, void** p, size_t bytes, cudaStream_t s);
 cudaError_t device_malloc(void** p, size_t bytes);  // cudaMalloc, for blocks that no pool should hold
 void* pinned_acquire(size_t bytes, size_t* capacity);  // null: out of memory

@@ -130,11 +130,15 @@ cudaError_t pool_acquire(cudaMemPool_t* pool) {
     return create_pool(~0ull, pool);  // hands nothing back on synchronisation
 }
 
-cudaError_t pool_shared(cudaMemPool_t* pool) {
+cudaError_t pool_shared(cudaMemPool_t* pool, bool* own) {
     *pool = nullptr;
+    *own = false;
     std::lock_guard<std::mutex> lk(kept_mutex());
     Kept* const k = kept();
-    if (!k) return cudaErrorInvalidDevice;
+    if (!k) {  // nothing is kept here
+        *own = true;
+        return create_pool(kKeepBytes, pool);
+    }
     if (!k->shared) {
         const cudaError_t e = create_pool(kKeepBytes, &k->shared);
         if (e != cudaSuccess) return e;

@@ -430,6 +430,7 @@ struct hlbm_server {
     cudaEvent_t fork_ev = nullptr, join_ev[kGraphBranches] = {};
     int device = 0;
     cudaMemPool_t pool = nullptr;  // device memory of the slots: the servers' pool (mem.cu)
+    bool own_pool = false;         // is it this server's alone?
     std::mutex mu;
     std::deque<Pending> waiting;
     std::vector<Live> live;
@@ -824,7 +825,7 @@ int hlbm_server_create(hlbm_server_t** out, size_t mem_budget, int storage, int 
     double feq[19];
     for (int i = 0; i < 19; ++i) feq[i] = feq_rest(i);
     cudaError_t e = cudaGetDevice(&s->device);
-    if (e == cudaSuccess) e = pool_shared(&s->pool);
+    if (e == cudaSuccess) e = pool_shared(&s->pool, &s->own_pool);
     if (e == cudaSuccess) e = cudaMalloc(&s->dtab, sizeof(DevTable));
     if (e == cudaSuccess && !(s->htab = static_cast<DevTable*>(pinned_acquire(sizeof(DevTable), &s->htab_bytes)))) e = cudaErrorMemoryAllocation;
     if (e == cudaSuccess) e = cudaMalloc(&s->dout, kMaxSlots * 8 * sizeof(double));
@@ -879,6 +880,7 @@ void hlbm_server_destroy(hlbm_server_t* s) {
     cudaFree(s->dtab);
     cudaFree(s->dout);
     cudaFree(s->dfeq);
+    if (s->own_pool && s->pool) cudaMemPoolDestroy(s->pool);
     pinned_release(s->htab, s->htab_bytes);
     pinned_release(s->hout, s->hout_bytes);
     delete s;

@@ -1,0 +1,126 @@
+// csrc/mem.cu on the CPU: the file is linked with the fake CUDA calls below, which know the
+// current context, what is allocated and what is freed. The argument names the case to run;
+// the exit status is 0 when it holds, and a line on stderr says what does not.
+#include <cuda_runtime.h>
+
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <set>
+
+#include "internal.h"
+
+namespace {
+
+unsigned long long g_context = 1;  // id of the current context
+bool g_have_ids = true;            // does the driver know context ids?
+std::map<char*, size_t> g_pinned;  // page-locked blocks that are allocated
+std::set<cudaMemPool_t> g_pools;   // pools that exist
+size_t g_next_pool = 16;
+int g_failed = 0;
+
+int fake_ctx_get_id(void*, unsigned long long* id) {
+    *id = g_context;
+    return g_context ? 0 : 201;
+}
+void expect(bool ok, const char* what) {
+    if (ok) return;
+    std::fprintf(stderr, "failed: %s\n", what);
+    g_failed = 1;
+}
+// Is [p, p + n) page-locked?
+bool mapped(const void* p, size_t n) {
+    const char* c = static_cast<const char*>(p);
+    for (const auto& b : g_pinned)
+        if (c >= b.first && c + n <= b.first + b.second) return true;
+    return false;
+}
+cudaError_t host_alloc(void** p, size_t n) {
+    *p = std::malloc(n);
+    g_pinned[static_cast<char*>(*p)] = n;
+    return cudaSuccess;
+}
+
+}  // namespace
+
+extern "C" {
+
+cudaError_t cudaGetDevice(int* d) {
+    *d = 0;
+    return cudaSuccess;
+}
+cudaError_t cudaGetLastError(void) { return cudaSuccess; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult* r) {
+    *f = g_have_ids ? reinterpret_cast<void*>(&fake_ctx_get_id) : nullptr;
+    *r = g_have_ids ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+    return g_have_ids ? cudaSuccess : cudaErrorSymbolNotFound;
+}
+cudaError_t cudaFree(void*) { return cudaSuccess; }
+cudaError_t cudaMalloc(void** p, size_t n) {
+    *p = std::malloc(n);
+    return cudaSuccess;
+}
+cudaError_t cudaMallocHost(void** p, size_t n) { return host_alloc(p, n); }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return host_alloc(p, n); }
+cudaError_t cudaFreeHost(void* p) {
+    const auto it = g_pinned.find(static_cast<char*>(p));
+    expect(it != g_pinned.end(), "only the start of an allocated page-locked block is freed");
+    if (it == g_pinned.end()) return cudaErrorInvalidValue;
+    std::free(p);
+    g_pinned.erase(it);
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*) {
+    *p = reinterpret_cast<cudaMemPool_t>(g_next_pool += 16);
+    g_pools.insert(*p);
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolDestroy(cudaMemPool_t p) {
+    expect(g_pools.erase(p) == 1, "only an existing pool is destroyed");
+    return cudaSuccess;
+}
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t p, size_t) {
+    expect(g_pools.count(p) == 1, "only an existing pool is trimmed");
+    return cudaSuccess;
+}
+cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) {
+    *p = std::malloc(n);
+    return cudaSuccess;
+}
+
+}  // extern "C"
+
+namespace {
+
+using namespace hlbm;
+
+// A driver without context ids: nothing can be kept, and everything still works.
+void no_context_ids() {
+    g_have_ids = false;
+    cudaMemPool_t a = nullptr, b = nullptr;
+    expect(pool_acquire(&a) == cudaSuccess && a, "a handle gets a pool");
+    bool own = false;
+    expect(pool_shared(&b, &own) == cudaSuccess && b && b != a && own, "a server gets a pool of its own");
+    if (own) cudaMemPoolDestroy(b);
+    pool_release(a);
+    size_t capacity = 0;
+    void* p = pinned_acquire(1000, &capacity);
+    expect(p && mapped(p, 1000), "a page-locked block");
+    pinned_release(p, capacity);
+    double* s = slot_acquire();
+    expect(s && mapped(s, 64), "a slot");
+    slot_release(s);
+    expect(g_pinned.empty() && g_pools.empty(), "everything is returned");
+}
+
+}  // namespace
+
+int main(int argc, char** argv) {
+    const char* const name = argc > 1 ? argv[1] : "";
+    if (!std::strcmp(name, "no_context_ids")) no_context_ids();
+    else expect(false, "a case of this program");
+    return g_failed;
+}
