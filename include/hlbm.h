@@ -116,8 +116,8 @@ int hlbm_create(hlbm_t** out, int velset, int nx, int ny, int nz, int storage, i
 
 /* Free the handle (after draining its stream). NULL is a no-op. Its device memory
  * goes back to the device except for up to 512 MiB, which stay mapped for the
- * next handle on that device (with the servers' memory at most 1.5 GiB per device
- * in all; hlbm_release_scratch, or a failed allocation, returns it). */
+ * next handle in that context (with the servers' memory at most 1.5 GiB per
+ * context in all; hlbm_release_scratch, or a failed allocation, returns it). */
 void hlbm_destroy(hlbm_t* h);
 
 /* Temporary device memory of the calls that need it (the checkpoints of
@@ -127,7 +127,7 @@ void hlbm_destroy(hlbm_t* h);
  * each synchronisation (re-mapping the 14.5 GB of checkpoints of a 128^3 x
  * 2000-step gradient took about 7 % of the call). This call waits for the
  * handle's stream and returns the pool's unused memory to the device, and with
- * it what is kept mapped for later handles and servers on the device; the
+ * it what is kept mapped for later handles and servers in the current context; the
  * next call that needs scratch maps it again. Not a paper operation (memory
  * management of this library). */
 int hlbm_release_scratch(hlbm_t* h);
@@ -391,8 +391,8 @@ int hlbm_server_info(hlbm_server_t* s, hlbm_server_stats* out);
  * device were out of memory (admission then backs off). */
 int hlbm_server_inject_alloc_failures(hlbm_server_t* s, int n);
 /* Free the server, its slots and its queued requests (results not polled are lost).
- * Up to 512 MiB of device memory per device, and 64 MiB of pinned host memory, stay
- * for later servers on that device (see hlbm_destroy). */
+ * Up to 512 MiB of device memory, and 64 MiB of pinned host memory, stay for later
+ * servers in that context (see hlbm_destroy). */
 void hlbm_server_destroy(hlbm_server_t* s);
 
 /* ---- allocation-free diagnostics --------------------------------------- */

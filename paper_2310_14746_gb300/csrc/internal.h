@@ -141,7 +141,7 @@ cudaError_t launch_fill_bytes0(void* p, size_t bytes, cudaStream_t s);
 
 size_t storage_bytes(int storage);
 
-// Memory kept between objects, on the current device (mem.cu). A pool belongs to one handle at
+// Memory kept between objects, in the current context (mem.cu). A pool belongs to one handle at
 // a time; every block taken from it is freed, and its streams are drained, before it is released.
 bool pool_keeps(size_t bytes);  // does a released pool keep this much mapped?
 cudaError_t pool_acquire(cudaMemPool_t* pool);

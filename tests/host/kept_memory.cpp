@@ -116,11 +116,61 @@ void no_context_ids() {
     expect(g_pinned.empty() && g_pools.empty(), "everything is returned");
 }
 
+// Objects of several contexts on one device, released in any order and with any context current.
+void several_contexts() {
+    double* const a = slot_acquire();
+    double* const b = slot_acquire();
+    cudaMemPool_t pool = nullptr, other = nullptr, again = nullptr;
+    pool_acquire(&pool);
+    pool_release(pool);
+    size_t ca = 0, cb = 0;
+    void* const pa = pinned_acquire(1000, &ca);
+    void* const pb = pinned_acquire(1000, &cb);
+    pinned_release(pa, ca);
+
+    g_context = 2;
+    double* const c = slot_acquire();
+    expect(c && c != a && c != b, "a slot of its own in the second context");
+    pool_acquire(&other);
+    expect(other != pool, "a pool of its own in the second context");
+    void* const pc = pinned_acquire(1000, &ca);
+    expect(pc != pa, "a page-locked block of its own in the second context");
+    pinned_release(pb, cb);  // of the first context
+
+    g_context = 1;
+    slot_release(a);
+    expect(mapped(b, 64) && mapped(c, 64), "the other handles keep their slots");
+    *b = 1.0;
+    pool_acquire(&again);
+    expect(again == pool, "the pool of the first context serves again");
+    pool_release(other);  // of the second context
+    expect(pool_acquire(&other) == cudaSuccess && g_pools.size() == 3, "and no pool of another one");
+    pool_release(other);
+    pool_release(again);
+    slot_release(c);
+    slot_release(b);
+    pinned_release(pc, ca);
+    expect(slot_acquire() == b && slot_acquire() == a, "released slots serve again");
+    void* const p1 = pinned_acquire(1000, &ca);
+    void* const p2 = pinned_acquire(1000, &cb);
+    expect((p1 == pa && p2 == pb) || (p1 == pb && p2 == pa), "blocks go back to the context that they come from");
+
+    for (g_context = 3; g_context < 10; ++g_context) {  // more contexts than are kept for
+        cudaMemPool_t p = nullptr;
+        double* const s = slot_acquire();
+        expect(pool_acquire(&p) == cudaSuccess && p && s && mapped(s, 64), "a handle in any context");
+        pool_release(p);
+        slot_release(s);
+    }
+    expect(g_pools.size() <= 2 * 4, "a bounded number of pools stays");
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
     const char* const name = argc > 1 ? argv[1] : "";
     if (!std::strcmp(name, "no_context_ids")) no_context_ids();
+    else if (!std::strcmp(name, "several_contexts")) several_contexts();
     else expect(false, "a case of this program");
     return g_failed;
 }
