@@ -16,10 +16,13 @@
 // request 1.2 -> 0.34 ms.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <set>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -36,7 +39,8 @@ constexpr size_t kSlotBytes = 64, kSlots = 256;  // small pinned results (one pa
 
 struct Kept {
     unsigned long long context = 0;  // id of the context that all of this belongs to; 0: a free record
-    std::vector<cudaMemPool_t> pools;
+    cudaMemPool_t pools[kKeepPools] = {};
+    size_t npools = 0;
     cudaMemPool_t shared = nullptr;
     std::multimap<size_t, void*> pinned;  // capacity -> block
     size_t pinned_bytes = 0;
@@ -45,8 +49,9 @@ struct Kept {
     std::vector<int> free_slots;
 };
 std::mutex& kept_mutex() {
-    static std::mutex* m = new std::mutex();
-    return *m;
+    static std::mutex m;
+    static_assert(std::is_trivially_destructible_v<std::mutex>, "usable while the process ends");
+    return m;
 }
 
 // 0: no context is current.
@@ -65,14 +70,27 @@ unsigned long long context_id() {
     return 0;
 }
 
+// Runs what may lack host memory for its bookkeeping. False: it did, and the object at hand is
+// then not kept (these functions are called from the C ABI, which no exception crosses).
+template <class Fn>
+bool has_memory(Fn&& fn) {
+    try {
+        fn();
+        return true;
+    } catch (const std::bad_alloc&) {
+        return false;
+    }
+}
+
 // All records, under kept_mutex(). Never destroyed (objects may be released while the process
 // ends), and a record stays its context's: an object may be released with another one current.
 struct Records {
     Kept of[kMaxDevices][kContexts];
 };
-Records& records() {
-    static Records* const all = new Records();
-    return *all;
+Records* records() {  // null: out of host memory
+    static Records* all = nullptr;
+    if (!all) all = new (std::nothrow) Records();
+    return all;
 }
 
 // What the current context keeps. Null: nothing can be kept.
@@ -80,26 +98,31 @@ Kept* kept() {
     int device = -1;
     if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= kMaxDevices) return nullptr;
     const unsigned long long id = context_id();
-    if (!id) return nullptr;
-    for (Kept& k : records().of[device]) {
-        if (!k.context) k.context = id;
+    Records* const all = id ? records() : nullptr;
+    if (!all) return nullptr;
+    for (Kept& k : all->of[device]) {
         if (k.context == id) return &k;
+        if (k.context) continue;
+        if (!has_memory([&] { k.free_slots.reserve(kSlots); })) return nullptr;
+        k.context = id;
+        return &k;
     }
     return nullptr;
 }
 
 // The record that a pool or pinned block is held under, which it is taken off; null: none.
 Kept* holder(void* p) {
-    for (auto& device : records().of)
-        for (Kept& k : device)
-            if (k.held.erase(p)) return &k;
+    if (Records* const all = records())
+        for (auto& device : all->of)
+            for (Kept& k : device)
+                if (k.held.erase(p)) return &k;
     return nullptr;
 }
 
 // Holds a new pool or pinned block under the current context.
 void hold(void* p) {
     holder(p);  // a context that is gone may have had one at this address
-    if (Kept* const k = kept()) k->held.insert(p);
+    if (Kept* const k = kept()) has_memory([&] { k->held.insert(p); });
 }
 
 cudaError_t create_pool(unsigned long long hold, cudaMemPool_t* pool) {
@@ -124,19 +147,21 @@ cudaError_t create_pool(unsigned long long hold, cudaMemPool_t* pool) {
 // All functions here work in the current context.
 
 void memory_give_back() {
-    std::vector<cudaMemPool_t> pools;
+    cudaMemPool_t pools[kKeepPools];
+    size_t npools = 0;
     std::multimap<size_t, void*> blocks;
     cudaMemPool_t shared = nullptr;
     {
         std::lock_guard<std::mutex> lk(kept_mutex());
         if (Kept* const k = kept()) {
-            pools.swap(k->pools);
+            std::swap(npools, k->npools);
+            std::copy(k->pools, k->pools + npools, pools);
             blocks.swap(k->pinned);
             k->pinned_bytes = 0;
             shared = k->shared;
         }
     }
-    for (cudaMemPool_t p : pools) cudaMemPoolDestroy(p);
+    for (size_t i = 0; i < npools; ++i) cudaMemPoolDestroy(pools[i]);
     if (shared) cudaMemPoolTrimTo(shared, 0);
     for (auto& b : blocks) cudaFreeHost(b.second);
 }
@@ -147,10 +172,9 @@ cudaError_t pool_acquire(cudaMemPool_t* pool) {
     {
         std::lock_guard<std::mutex> lk(kept_mutex());
         Kept* const k = kept();
-        if (k && !k->pools.empty()) {
-            *pool = k->pools.back();
-            k->pools.pop_back();
-            k->held.insert(*pool);
+        if (k && k->npools) {
+            *pool = k->pools[--k->npools];
+            has_memory([&] { k->held.insert(*pool); });
             return cudaSuccess;
         }
     }
@@ -184,8 +208,8 @@ void pool_release(cudaMemPool_t pool) {
     {
         std::lock_guard<std::mutex> lk(kept_mutex());
         Kept* const k = holder(pool);
-        if (trimmed && k && k->pools.size() < kKeepPools) {
-            k->pools.push_back(pool);
+        if (trimmed && k && k->npools < kKeepPools) {
+            k->pools[k->npools++] = pool;
             return;
         }
     }
@@ -222,7 +246,7 @@ void* pinned_acquire(size_t bytes, size_t* capacity) {
                 *capacity = it->first;
                 k->pinned_bytes -= it->first;
                 k->pinned.erase(it);
-                k->held.insert(b);
+                has_memory([&] { k->held.insert(b); });
                 return b;
             }
         }
@@ -249,8 +273,7 @@ void pinned_release(void* b, size_t capacity) {
     {
         std::lock_guard<std::mutex> lk(kept_mutex());
         Kept* const k = holder(b);
-        if (k && k->pinned_bytes + capacity <= kKeepPinned) {
-            k->pinned.emplace(capacity, b);
+        if (k && k->pinned_bytes + capacity <= kKeepPinned && has_memory([&] { k->pinned.emplace(capacity, b); })) {
             k->pinned_bytes += capacity;
             return;
         }
@@ -284,8 +307,9 @@ void slot_release(double* p) {
     char* const c = reinterpret_cast<char*>(p);
     {
         std::lock_guard<std::mutex> lk(kept_mutex());
-        for (auto& device : records().of)
-            for (Kept& k : device)
+        Records* const all = records();
+        for (int d = 0; all && d < kMaxDevices; ++d)
+            for (Kept& k : all->of[d])
                 if (k.slots && c >= k.slots && c < k.slots + kSlotBytes * kSlots) {  // never freed: others use the block
                     k.free_slots.push_back((int)((c - k.slots) / kSlotBytes));
                     return;

@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
 #include <set>
 
 #include "internal.h"
@@ -19,6 +20,7 @@ std::map<char*, size_t> g_pinned;  // page-locked blocks that are allocated
 std::set<cudaMemPool_t> g_pools;   // pools that exist
 size_t g_next_pool = 16;
 int g_failed = 0;
+bool g_no_memory = false;  // operator new fails
 
 int fake_ctx_get_id(void*, unsigned long long* id) {
     *id = g_context;
@@ -37,12 +39,23 @@ bool mapped(const void* p, size_t n) {
     return false;
 }
 cudaError_t host_alloc(void** p, size_t n) {
+    const bool no_memory = g_no_memory;
+    g_no_memory = false;  // for the list below
     *p = std::malloc(n);
     g_pinned[static_cast<char*>(*p)] = n;
+    g_no_memory = no_memory;
     return cudaSuccess;
 }
 
 }  // namespace
+
+void* operator new(size_t n) {
+    if (g_no_memory) throw std::bad_alloc();
+    return std::malloc(n ? n : 1);
+}
+void* operator new(size_t n, const std::nothrow_t&) noexcept { return g_no_memory ? nullptr : std::malloc(n ? n : 1); }
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, size_t) noexcept { std::free(p); }
 
 extern "C" {
 
@@ -73,8 +86,11 @@ cudaError_t cudaFreeHost(void* p) {
     return cudaSuccess;
 }
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*) {
+    const bool no_memory = g_no_memory;
+    g_no_memory = false;
     *p = reinterpret_cast<cudaMemPool_t>(g_next_pool += 16);
     g_pools.insert(*p);
+    g_no_memory = no_memory;
     return cudaSuccess;
 }
 cudaError_t cudaMemPoolDestroy(cudaMemPool_t p) {
@@ -165,12 +181,38 @@ void several_contexts() {
     expect(g_pools.size() <= 2 * 4, "a bounded number of pools stays");
 }
 
+// Host memory runs out at any call: nothing is thrown, and what cannot be kept is freed.
+void no_host_memory() {
+    for (int fail_from = 0; fail_from < 4; ++fail_from) {
+        g_no_memory = fail_from == 0;
+        cudaMemPool_t p = nullptr;
+        size_t capacity = 0;
+        bool own = false;
+        cudaMemPool_t shared = nullptr;
+        expect(pool_shared(&shared, &own) == cudaSuccess, "a server gets a pool");
+        if (own) cudaMemPoolDestroy(shared);
+        g_no_memory = fail_from <= 1;
+        expect(pool_acquire(&p) == cudaSuccess, "a handle gets a pool");
+        void* const b = pinned_acquire(1000, &capacity);
+        double* const s = slot_acquire();
+        expect(b && mapped(b, 1000) && s && mapped(s, 64), "and page-locked memory");
+        g_no_memory = fail_from <= 2;
+        pool_release(p);
+        pinned_release(b, capacity);
+        slot_release(s);
+        memory_give_back();
+    }
+    g_no_memory = false;
+    expect(g_pools.size() == 1 && g_pinned.size() == 1, "the servers' pool and the slots stay, nothing else");
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
     const char* const name = argc > 1 ? argv[1] : "";
     if (!std::strcmp(name, "no_context_ids")) no_context_ids();
     else if (!std::strcmp(name, "several_contexts")) several_contexts();
+    else if (!std::strcmp(name, "no_host_memory")) no_host_memory();
     else expect(false, "a case of this program");
     return g_failed;
 }
