@@ -82,11 +82,51 @@ __device__ __forceinline__ void chain_wait(int& x) {
 // with walls 113 -> 102, 221x143x203 163 -> 159, 256^3 376.6 -> 373.4, 128^3 49.4 ->
 // 49.5, 64^3 5.81 -> 5.46, 48^3 4.10 -> 3.84, 33x41x44 4.04 -> 3.33; FP16 152x104x96
 // with walls 41.2 -> 35.9. Equal pieces with as many idle lanes measured 4 % slower
-// (D2Q9 329x245), so a tie keeps the old shape.
-inline dim3 row_block(int nx) {
+// (D2Q9 329x245), so a tie keeps the old shape. So does a y axis that the rows of this rule
+// would not cover with one grid: a server's lattice may have up to 131070 rows of more than 64
+// cells, 262140 of up to 64 and 524280 of up to 32.
+constexpr int kMaxGridY = 65535;
+inline dim3 row_block(int nx, int ny) {
     const int pieces = (nx + 255) / 256, bx = ((nx + pieces - 1) / pieces + 31) / 32 * 32;
-    if (pieces > 1 && pieces * bx >= (nx + 127) / 128 * 128) return dim3(128, 2, 1);
-    return dim3(bx, bx >= 128 ? 1 : 128 / bx, 1);
+    const int old_bx = nx > 96 ? 128 : (nx + 31) / 32 * 32;
+    const dim3 old(old_bx, 256 / old_bx, 1), blk(bx, bx >= 128 ? 1 : 128 / bx, 1);
+    if (pieces > 1 && pieces * bx >= (nx + 127) / 128 * 128) return old;
+    return (ny + (int)blk.y - 1) / (int)blk.y > kMaxGridY ? old : blk;
+}
+
+// Block of a paired kernel (x in cell pairs): about 128 threads that leave the fewest
+// idle lanes over the lattice, counting the row tail, the partly filled warp of a
+// block and the tail of y. Candidate widths: 64, 32 and 16 pairs, and the row cut into
+// one to four equal pieces (any width: a warp may span rows). Before, blocks had 256
+// threads and widths of 32, 64, 96 or 128 pairs. Measured, us per step before -> with
+// this rule: two-lattice FP16 96^3 15.4 -> 12.0, 160^3 63.1 -> 55.8, 42x50x60 4.35 ->
+// 3.59, 64^3 5.12 -> 4.61, 192^3 94.5 -> 92.8, 256^3 216.3 -> 214.1, 384x192x192 184.4 ->
+// 182.0; BF16 160^3 57.3 -> 53.2, 176x176x152 (drag) 70.9 -> 67.8, 204x190x180 (tensor)
+// 131 -> 126; in place FP16 80x64x72 8.7 -> 6.2, 160^3 63.7 -> 57.6, BF16 192^3 95.5 ->
+// 93.8. Pieces of 16 pairs where nx is no multiple of 32 measured 110 instead of 91.8
+// (BF16 222x144x200), hence the penalty. Where y is longer than a grid, only blocks of
+// enough rows count (16 pairs times 8 rows always fit up to 524280 rows).
+inline dim3 pair_block(int nx, int ny, int cap) {
+    const int pairs = nx / 2, most = cap < 192 ? cap : 192;
+    const int widths[] = {64, 32, 16, pairs, (pairs + 1) / 2, (pairs + 2) / 3, (pairs + 3) / 4};
+    dim3 best(32, 4, 1);
+    double score_best = -1.0;
+    for (int bx : widths) {
+        if (bx < 1 || bx > most) continue;
+        for (int by = 1; bx * by <= most; ++by) {
+            if ((ny + by - 1) / by > kMaxGridY) continue;
+            const int threads = bx * by, lanes = (threads + 31) / 32 * 32;
+            double score = (double)pairs / ((pairs + bx - 1) / bx) * by / lanes * ny / ((ny + by - 1) / by * by);
+            if (threads < 64) score *= 0.8;            // too few warps per block to fill an SM
+            if (bx < 32 && bx < pairs) score *= nx % 32 == 0 ? 0.97 : 0.85;  // short pieces, worse when they straddle lines
+            score -= 1e-4 * (threads < 128 ? 128 - threads : threads - 128) / 128;
+            if (score > score_best) {
+                score_best = score;
+                best = dim3(bx, by, 1);
+            }
+        }
+    }
+    return best;
 }
 
 // Solid-link masks from a solid flag per cell (uint8, nonzero = solid): bit i of

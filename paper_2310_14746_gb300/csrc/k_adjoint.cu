@@ -191,7 +191,7 @@ static cudaError_t adjoint_impl(const LaunchCtx& c, const void* fn, const float*
     using C = typename S::C;
     const Geometry g = geom(c);
     const Phys<C> ph = make_phys<C, Q>(c.tau, c.F);
-    const dim3 blk = row_block(c.nx);
+    const dim3 blk = row_block(c.nx, c.ny);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     const auto* f = static_cast<const typename S::T*>(fn);
     if ((size_t)Q * g.N < ((size_t)1 << 31))
@@ -230,7 +230,7 @@ cudaError_t launch_adjoint_step(const LaunchCtx& c, const void* fn, const float*
 
 cudaError_t launch_flux_seed(const LaunchCtx& c, float* lam, int plane_x) {
     const Geometry g = geom(c);
-    const dim3 blk = row_block(c.nx);
+    const dim3 blk = row_block(c.nx, c.ny);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     const bool walls = c.wall[0] || c.wall[1] || c.wall[2];
     if (c.q == 9) {

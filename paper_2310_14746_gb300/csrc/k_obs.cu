@@ -45,7 +45,7 @@ template <int Q, class S, bool WALLS>
 static cudaError_t moments_impl(const LaunchCtx& c, int lay, const void* f, void* rho, void* u, int f64) {
     using C = typename S::C;
     const Geometry g = geom(c);
-    const dim3 blk = row_block(c.nx);
+    const dim3 blk = row_block(c.nx, c.ny);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     const auto* a = static_cast<const typename S::T*>(f);
     with_layout((size_t)Q * g.N, lay, [&]<int LAY>() {
@@ -157,7 +157,7 @@ k_fill_state(const double* fnat, int lay, Geometry g, typename S::C s, typename 
 template <int Q, class S, bool WALLS>
 static cudaError_t write_impl(const LaunchCtx& c, int lay, const double* fnat, int uniform, void* f) {
     using C = typename S::C;
-    const dim3 blk = row_block(c.nx);
+    const dim3 blk = row_block(c.nx, c.ny);
     if (uniform) {
         const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, (c.nz + kFillZ - 1) / kFillZ);
         k_fill_state<Q, S, WALLS><<<grd, blk, 0, c.stream>>>(fnat, lay, geom(c), C(c.scale),
@@ -173,7 +173,7 @@ static cudaError_t write_impl(const LaunchCtx& c, int lay, const double* fnat, i
 template <int Q, class S, bool WALLS>
 static cudaError_t read_impl(const LaunchCtx& c, int lay, const void* f, double* fnat) {
     using C = typename S::C;
-    const dim3 blk = row_block(c.nx);
+    const dim3 blk = row_block(c.nx, c.ny);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     with_layout((size_t)Q * c.nx * c.ny * c.nz, lay, [&]<int LAY>() {
         k_read_state<Q, S, WALLS, LAY><<<grd, blk, 0, c.stream>>>(static_cast<const typename S::T*>(f), lay, geom(c),

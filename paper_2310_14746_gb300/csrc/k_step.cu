@@ -32,7 +32,7 @@ __global__ void k_build_links(const unsigned char* __restrict__ solid, unsigned*
 
 cudaError_t launch_build_links(const LaunchCtx& c, const unsigned char* solid, unsigned* links) {
     Geometry g{c.nx, c.ny, c.nz, c.wall[0], c.wall[1], c.wall[2], (size_t)c.nx * c.ny * c.nz};
-    const dim3 blk = row_block(c.nx);
+    const dim3 blk = row_block(c.nx, c.ny);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     if (c.q == 9) k_build_links<9><<<grd, blk, 0, c.stream>>>(solid, links, g);
     else k_build_links<19><<<grd, blk, 0, c.stream>>>(solid, links, g);

@@ -116,7 +116,7 @@ cudaError_t step_impl(const LaunchCtx& c, int mode, const void* fin, void* fout,
     using T = typename S::T;
     Geometry g{c.nx, c.ny, c.nz, c.wall[0], c.wall[1], c.wall[2], (size_t)c.nx * c.ny * c.nz};
     const Phys<C> ph = make_phys<C, Q>(c.tau, c.F);
-    const dim3 blk = S::kind == 0 ? step_block_f64(c.nx, c.ny) : row_block(c.nx);
+    const dim3 blk = S::kind == 0 ? step_block_f64(c.nx, c.ny) : row_block(c.nx, c.ny);
     const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
     const C s = C(c.scale), inv_s = C(1.0 / c.scale);
     Planes<const T, Q> a;
