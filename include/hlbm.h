@@ -375,7 +375,9 @@ int hlbm_server_set_refinement(hlbm_server_t* s, int enable, double floor_coef);
  * do not depend on it, only when they arrive. */
 int hlbm_server_set_priority(hlbm_server_t* s, double backfill);
 /* Queue a request (validated and copied); *id receives its identifier.
- * HLBM_ERR_OOM if it could never fit the budget. */
+ * HLBM_ERR_OOM if it could never fit the budget. Limits of the launch grids
+ * (HLBM_ERR_INVALID_ARG beyond them): ny <= 131070 for nx > 64, 262140 for
+ * nx > 32, 524280 otherwise; nz <= 65535 with u_out or at least 2^18 cells. */
 int hlbm_server_submit(hlbm_server_t* s, const hlbm_request* r, uint64_t* id);
 /* One scheduling round: admit, run check_every steps of this round's slots
  * (see hlbm_server_set_priority), check them, retire. Synchronises. *active / *waiting (may be NULL) receive the

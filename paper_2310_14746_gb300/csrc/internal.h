@@ -85,11 +85,15 @@ __device__ __forceinline__ void chain_wait(int& x) {
 // (D2Q9 329x245), so a tie keeps the old shape. So does a y axis that the rows of this rule
 // would not cover with one grid: a server's lattice may have up to 131070 rows of more than 64
 // cells, 262140 of up to 64 and 524280 of up to 32.
-constexpr int kMaxGridY = 65535;
+constexpr int kMaxGridY = 65535, kMaxGridZ = 65535;
+inline dim3 row_block_old(int nx) {
+    const int bx = nx > 96 ? 128 : (nx + 31) / 32 * 32;
+    return dim3(bx, 256 / bx, 1);
+}
+inline long long rows_per_grid(int nx) { return (long long)kMaxGridY * row_block_old(nx).y; }
 inline dim3 row_block(int nx, int ny) {
     const int pieces = (nx + 255) / 256, bx = ((nx + pieces - 1) / pieces + 31) / 32 * 32;
-    const int old_bx = nx > 96 ? 128 : (nx + 31) / 32 * 32;
-    const dim3 old(old_bx, 256 / old_bx, 1), blk(bx, bx >= 128 ? 1 : 128 / bx, 1);
+    const dim3 old = row_block_old(nx), blk(bx, bx >= 128 ? 1 : 128 / bx, 1);
     if (pieces > 1 && pieces * bx >= (nx + 127) / 128 * 128) return old;
     return (ny + (int)blk.y - 1) / (int)blk.y > kMaxGridY ? old : blk;
 }

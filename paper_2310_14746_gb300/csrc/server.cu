@@ -894,6 +894,10 @@ int hlbm_server_submit(hlbm_server_t* s, const hlbm_request* r, uint64_t* id) {
     if (!(r->tol > 0.0) || r->max_steps < 1) return HLBM_ERR_INVALID_ARG;
     const size_t n = (size_t)r->nx * r->ny * r->nz;
     if (n > ((size_t)1 << 31) / 19) return HLBM_ERR_INVALID_ARG;
+    // what no launch grid covers would fail in every round: the initial state (eight planes per
+    // block), and one plane per block in a direct slot's steps and in the moments for u_out
+    if (r->ny > rows_per_grid(r->nx)) return HLBM_ERR_INVALID_ARG;
+    if (r->nz > kMaxGridZ && (n >= kDirectCells || r->u_out)) return HLBM_ERR_INVALID_ARG;
     if (!host_unit_interval(r->varpi, n)) return HLBM_ERR_INVALID_ARG;
     if (s->slot_bytes(*r) > s->budget) return HLBM_ERR_OOM;
     Pending p;

@@ -35,3 +35,21 @@ def test_tall_request(nx, ny, storage):
     one = _solve(vp, storage)
     tall = _solve(np.ascontiguousarray(np.tile(vp, (1, 10, 1))), storage)
     np.testing.assert_array_equal(tall, np.tile(one, (1, 1, 10, 1)))
+
+
+def test_requests_beyond_the_grids_are_refused():
+    """What no launch grid covers is refused when submitted, and the server goes on; the largest
+    axes that are covered run."""
+    srv = Server(4 << 30, hb.HLBM_F32, 10)
+    kw = dict(tau=0.7, F=(1e-4, 0, 0), tol=1e-30, max_steps=10)
+    for shape, want_u in (((1, 131071, 65), False), ((1, 262141, 33), False), ((1, 524281, 1), False),
+                          ((65536, 2, 2), False), ((300000, 1, 1), False), ((65536, 1, 1), True)):
+        with pytest.raises(hb.HlbmError) as e:
+            srv.submit(np.full(shape, 0.5, np.float32), want_u=want_u, **kw)
+        assert e.value.status == hb.HLBM_ERR_INVALID_ARG
+    taken = [srv.submit(np.full(shape, 0.5, np.float32), want_u=want_u, **kw)
+             for shape, want_u in (((1, 131070, 65), True), ((1, 524280, 1), True), ((65535, 2, 2), True), ((65536, 1, 2), False))]
+    done = srv.run_until_idle()
+    srv.close()
+    assert sorted(r["id"] for r in done) == sorted(taken)
+    assert all(r["steps"] == 10 for r in done)
