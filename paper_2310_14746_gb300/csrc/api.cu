@@ -53,7 +53,8 @@ struct hlbm_lattice {
     int q = 19, nx = 0, ny = 0, nz = 0, storage = HLBM_F32, pattern = HLBM_TWO_LATTICE;
     int device = 0;
     cudaStream_t stream = nullptr;
-    cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
+    cudaStream_t own_stream = nullptr;  // of the handle alone: graphs are captured there, and gradients run there
+    cudaEvent_t own_ev = nullptr;
     double tau = 1.0;
     double F[3] = {0.0, 0.0, 0.0};
     int bc[3] = {HLBM_PERIODIC, HLBM_PERIODIC, HLBM_PERIODIC};
@@ -160,7 +161,8 @@ void free_all(hlbm_t* h) {
     for (cudaEvent_t e : h->series_ev)
         if (e) cudaEventDestroy(e);
     if (h->series_stream) cudaStreamDestroy(h->series_stream);
-    if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
+    if (h->own_ev) cudaEventDestroy(h->own_ev);
+    if (h->own_stream) cudaStreamDestroy(h->own_stream);
     void* const blocks[] = {h->buf[0], h->buf[1], h->varpi, h->u_prev, h->partials, h->out8};
     for (void* p : blocks)
         if (p && (!h->pooled || cudaFreeAsync(p, h->stream) != cudaSuccess)) cudaFree(p);
@@ -200,16 +202,16 @@ int steps_on(hlbm_t* h, cudaStream_t s, long n, bool two) {
 
 bool at_graph_origin(const hlbm_t* h) { return h->pattern == HLBM_TWO_LATTICE ? h->cur == 0 : h->aa_odd == 0; }
 
-// Capture what `body` launches on the handle's capture stream, starting from the graph origin layout,
+// Capture what `body` launches on the handle's own stream, starting from the graph origin layout,
 // which an even number of steps returns to.
 template <class Body>
 int capture(hlbm_t* h, cudaGraphExec_t* exec, Body&& body) {
-    if (!h->cap_stream) HLBM_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
+    if (!h->own_stream) HLBM_CUDA(cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking));
     const int cur0 = h->cur, odd0 = h->aa_odd;
     cudaGraph_t graph = nullptr;
-    HLBM_CUDA(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = body(h->cap_stream);
-    cudaError_t e = cudaStreamEndCapture(h->cap_stream, &graph);
+    HLBM_CUDA(cudaStreamBeginCapture(h->own_stream, cudaStreamCaptureModeThreadLocal));
+    const int rc = body(h->own_stream);
+    cudaError_t e = cudaStreamEndCapture(h->own_stream, &graph);
     h->cur = cur0;
     h->aa_odd = odd0;
     if (rc != HLBM_OK) {
@@ -814,31 +816,47 @@ struct Scratch {
     }
 };
 
-// Copy the current state into `dst` in the NATURAL layout.
-int copy_natural(hlbm_t* h, void* dst, Scratch& sc) {
+// The handle's own stream for the length of a call, behind what its stream holds so far. Chained
+// kernels (launch_chained) must follow one another directly: on the caller's stream another thread,
+// with a handle of its own, can put a copy or a graph between two of them, and here nobody can.
+// Waited for at the latest when the call ends, before its scratch is given back.
+struct OwnStream {
+    hlbm_t* h;
+    explicit OwnStream(hlbm_t* hh) : h(hh) {}
+    ~OwnStream() {
+        if (h->own_stream) cudaStreamSynchronize(h->own_stream);
+    }
+    cudaError_t fork() {
+        cudaError_t e = cudaSuccess;
+        if (!h->own_stream) e = cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking);
+        if (e == cudaSuccess && !h->own_ev) e = cudaEventCreateWithFlags(&h->own_ev, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(h->own_ev, h->stream);
+        return e == cudaSuccess ? cudaStreamWaitEvent(h->own_stream, h->own_ev, 0) : e;
+    }
+};
+
+// Copy the current state into `dst` in the NATURAL layout, on c's stream. tmp: q doubles per
+// cell, for the in-place pattern.
+int copy_natural(hlbm_t* h, const LaunchCtx& c, void* dst, double* tmp) {
     if (h->pattern == HLBM_TWO_LATTICE) {
-        HLBM_CUDA(cudaMemcpyAsync(dst, h->state(), h->state_bytes(), cudaMemcpyDeviceToDevice, h->stream));
+        HLBM_CUDA(cudaMemcpyAsync(dst, h->state(), h->state_bytes(), cudaMemcpyDeviceToDevice, c.stream));
         return HLBM_OK;
     }
-    double* tmp = nullptr;
-    HLBM_CUDA(sc.alloc((void**)&tmp, (size_t)h->q * h->cells * sizeof(double)));
-    HLBM_CUDA(launch_read_state(h->ctx(h->stream), h->layout(), h->state(), tmp));
-    HLBM_CUDA(launch_write_state(h->ctx(h->stream), kNatural, tmp, 0, dst));
+    HLBM_CUDA(launch_read_state(c, h->layout(), h->state(), tmp));
+    HLBM_CUDA(launch_write_state(c, kNatural, tmp, 0, dst));
     return HLBM_OK;
 }
 
-// Make a NATURAL-layout buffer the handle's state.
-int adopt_natural(hlbm_t* h, const void* src, Scratch& sc) {
+// Make a NATURAL-layout buffer the handle's state, on c's stream.
+int adopt_natural(hlbm_t* h, const LaunchCtx& c, const void* src, double* tmp) {
     if (h->pattern == HLBM_TWO_LATTICE) {
-        HLBM_CUDA(cudaMemcpyAsync(h->buf[0], src, h->state_bytes(), cudaMemcpyDeviceToDevice, h->stream));
+        HLBM_CUDA(cudaMemcpyAsync(h->buf[0], src, h->state_bytes(), cudaMemcpyDeviceToDevice, c.stream));
         h->cur = 0;
         return HLBM_OK;
     }
-    double* tmp = nullptr;
-    HLBM_CUDA(sc.alloc((void**)&tmp, (size_t)h->q * h->cells * sizeof(double)));
-    HLBM_CUDA(launch_read_state(h->ctx(h->stream), kNatural, src, tmp));
+    HLBM_CUDA(launch_read_state(c, kNatural, src, tmp));
     h->aa_odd = 0;
-    HLBM_CUDA(launch_write_state(h->ctx(h->stream), h->layout(), tmp, 0, h->buf[0]));
+    HLBM_CUDA(launch_write_state(c, h->layout(), tmp, 0, h->buf[0]));
     return HLBM_OK;
 }
 
@@ -858,21 +876,25 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
     Scratch sc(h);
     char *snaps = nullptr, *seg = nullptr;
     float *lam_a = nullptr, *lam_b = nullptr, *gacc = nullptr;
-    double* jdev = nullptr;
+    double *jdev = nullptr, *tmp = nullptr;
     HLBM_CUDA(sc.alloc((void**)&snaps, sb * nsnap));
     HLBM_CUDA(sc.alloc((void**)&seg, sb * nseg));
     HLBM_CUDA(sc.alloc((void**)&lam_a, (size_t)h->q * N * sizeof(float)));
     HLBM_CUDA(sc.alloc((void**)&lam_b, (size_t)h->q * N * sizeof(float)));
     HLBM_CUDA(sc.alloc((void**)&gacc, N * sizeof(float)));
     HLBM_CUDA(sc.alloc((void**)&jdev, sizeof(double)));
-    int rc = copy_natural(h, snaps, sc);
+    if (h->pattern != HLBM_TWO_LATTICE) HLBM_CUDA(sc.alloc((void**)&tmp, (size_t)h->q * N * sizeof(double)));
+    OwnStream own(h);
+    HLBM_CUDA(own.fork());
+    c.stream = h->own_stream;
+    int rc = copy_natural(h, c, snaps, tmp);
     if (rc != HLBM_OK) return rc;
 
     // forward sweep, keeping f^{k*every}, and in the last segment every state: the reverse sweep
     // starts there, so only the segments before it are recomputed (90 steps kept every 45: 134
     // forward steps instead of 178). The final state goes to slot 0, which no segment uses.
-    // Where nothing needs the state in between, two steps go in one launch, and all kernels are
-    // chained (180 steps of 128^3 kept every 45: 30.4 -> 28.8 ms for the gradient).
+    // Where nothing needs the state in between, two steps go in one launch; the single steps and the
+    // reverse steps are chained (180 steps of 128^3 kept every 45: 30.4 -> 28.8 ms for the gradient).
     const long last0 = (nsnap - 1) * every;
     const bool two = step2_applies(c);
     void* a = snaps;
@@ -890,12 +912,12 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
     }
     c.chained = CHAIN_NONE;
     HLBM_CUDA(launch_plane_flux(c, kNatural, a, plane_x, jdev));
-    rc = adopt_natural(h, a, sc);
+    rc = adopt_natural(h, c, a, tmp);
     if (rc != HLBM_OK) return rc;
 
     // reverse sweep
     HLBM_CUDA(launch_flux_seed(c, lam_a, plane_x));
-    HLBM_CUDA(cudaMemsetAsync(gacc, 0, N * sizeof(float), h->stream));
+    HLBM_CUDA(cudaMemsetAsync(gacc, 0, N * sizeof(float), c.stream));
     for (long sg = nsnap - 1; sg >= 0 && nsteps > 0; --sg) {
         const long s0 = sg * every;
         const long s1 = s0 + every < nsteps ? s0 + every : nsteps;
@@ -911,9 +933,9 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
         }
     }
     HLBM_CUDA(cudaMemcpyAsync(grad, gacc, N * sizeof(float),
-                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
-    HLBM_CUDA(cudaMemcpyAsync(J, jdev, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    HLBM_CUDA(cudaStreamSynchronize(h->stream));
+                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c.stream));
+    HLBM_CUDA(cudaMemcpyAsync(J, jdev, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+    HLBM_CUDA(cudaStreamSynchronize(c.stream));
     h->step += nsteps;
     return HLBM_OK;
 }
