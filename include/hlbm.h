@@ -157,7 +157,8 @@ int hlbm_set_porosity(hlbm_t* h, const float* varpi, int on_device);
  * surface); solid cells are not updated and report rho = 1, u = 0 (and rest
  * populations from hlbm_get_populations). With varpi = 1 in the fluid this is
  * the pore-scale problem whose permeability the homogenized field stands in
- * for (Thm. thmStatNSECase4). NULL removes the obstacles. Set the domain
+ * for (Thm. thmStatNSECase4). NULL removes the obstacles: their cells become
+ * fluid at rest (the in-place pattern needs scratch for it). Set the domain
  * boundaries first (hlbm_set_boundary returns HLBM_ERR_STATE while a mask is
  * set); the post-collision state of the fluid cells is kept across the call.
  * Not supported by hlbm_adjoint_flux_grad (HLBM_ERR_STATE). Synchronises. */

@@ -283,6 +283,15 @@ int reset_counters(hlbm_t* h) {
     return HLBM_OK;
 }
 
+// The solid cells rest in every buffer: steps leave them alone, so they would otherwise hold what
+// the memory held before, and show it in a checkpoint or once the mask is removed.
+cudaError_t rest_solids(hlbm_t* h) {
+    cudaError_t e = cudaSuccess;
+    for (void* b : h->buf)
+        if (b && h->links && e == cudaSuccess) e = launch_rest_solid(h->ctx(h->stream), b);
+    return e;
+}
+
 // Write natural FP64 populations (device pointer; q values if uniform) as the new state.
 int write_state(hlbm_t* h, const double* fnat_dev, int uniform) {
     h->cur = 0;
@@ -560,7 +569,17 @@ int hlbm_set_solid_mask(hlbm_t* h, const unsigned char* solid, int on_device) {
     DeviceGuard g(h->device);
     if (!solid) {  // remove the obstacles
         if (h->links) {
-            HLBM_CUDA(cudaStreamSynchronize(h->stream));
+            // in place, populations that bounced off a solid cell lie elsewhere than ones that
+            // travelled on: re-lay the state (two lattices hold it unstreamed)
+            double* nat = nullptr;
+            if (h->pattern != HLBM_TWO_LATTICE) HLBM_CUDA(scratch_alloc(h, (void**)&nat, (size_t)h->q * h->cells * sizeof(double)));
+            LaunchCtx c = h->ctx(h->stream);
+            cudaError_t e = nat ? launch_read_state(c, h->layout(), h->state(), nat) : cudaSuccess;
+            c.links = nullptr;
+            if (nat && e == cudaSuccess) e = launch_write_state(c, h->layout(), nat, 0, h->state());
+            if (nat) cudaFreeAsync(nat, h->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+            if (e != cudaSuccess) return cuda_fail(e);
             cudaFree(h->links);
             h->links = nullptr;
         }
@@ -578,6 +597,7 @@ int hlbm_set_solid_mask(hlbm_t* h, const unsigned char* solid, int on_device) {
     if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(dsolid, solid, h->cells, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = launch_build_links(h->ctx(h->stream), on_device ? solid : dsolid, h->links);
     if (e == cudaSuccess) e = launch_write_state(h->ctx(h->stream), h->layout(), tmp, 0, h->state());
+    if (e == cudaSuccess) e = rest_solids(h);
     if (dsolid) cudaFreeAsync(dsolid, h->stream);
     cudaFreeAsync(tmp, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -1004,6 +1024,7 @@ int hlbm_load(hlbm_t* h, const char* path) {
     h->settings_changed();
     HLBM_CUDA(cudaMemcpyAsync(h->buf[0], st.data(), st.size(), cudaMemcpyHostToDevice, h->stream));
     HLBM_CUDA(cudaMemcpyAsync(h->varpi, vp.data(), vp.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream));
+    HLBM_CUDA(rest_solids(h));
     HLBM_CUDA(cudaMemsetAsync(h->u_prev, 0, 3 * h->cells * h->arith_bytes(), h->stream));
     HLBM_CUDA(cudaStreamSynchronize(h->stream));
     return HLBM_OK;

@@ -175,6 +175,8 @@ cudaError_t launch_reduce(const LaunchCtx& c, int layout, const void* f, void* u
 // values applied to every cell when uniform == 1.
 cudaError_t launch_write_state(const LaunchCtx& c, int layout, const double* fnat, int uniform,
                                void* f);
+// Rest populations into the solid cells (c.links) of a state buffer in any layout.
+cudaError_t launch_rest_solid(const LaunchCtx& c, void* f);
 // Read the state as natural FP64 full populations [q][cells].
 cudaError_t launch_read_state(const LaunchCtx& c, int layout, const void* f, double* fnat);
 

@@ -83,6 +83,20 @@ k_write_state(const double* fnat, int uniform, int lay, Geometry g, typename S::
     }
 }
 
+// Rest populations (deviation 0) into the slots of the solid cells, which are theirs alone in every
+// layout: no step reads or writes them, so they keep what this kernel leaves.
+template <int Q, class S>
+__global__ void __launch_bounds__(256) k_rest_solid(typename S::T* f, Geometry g, const unsigned* links) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int z = blockIdx.z;
+    if (x >= g.nx || y >= g.ny) return;
+    const size_t cell = (size_t)x + (size_t)g.nx * ((size_t)y + (size_t)g.ny * (size_t)z);
+    if (!(links[cell] & kSolidBit)) return;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[(size_t)i * g.N + cell] = typename S::T(0.0f);
+}
+
 // float -> double, exactly, on the integer pipe: a conversion instruction runs on the
 // FP64 pipe, which the addition of the weight below already keeps busy (two lanes
 // per clock and SM). Zero and normal values; the others take the instruction.
@@ -192,6 +206,15 @@ cudaError_t launch_write_state(const LaunchCtx& c, int layout, const double* fna
 
 cudaError_t launch_read_state(const LaunchCtx& c, int layout, const void* f, double* fnat) {
     return dispatch(c, [&]<int Q, class S, bool W>() { return read_impl<Q, S, W>(c, layout, f, fnat); });
+}
+
+cudaError_t launch_rest_solid(const LaunchCtx& c, void* f) {
+    return dispatch(c, [&]<int Q, class S, bool W>() {
+        const dim3 blk = row_block(c.nx, c.ny);
+        const dim3 grd((c.nx + blk.x - 1) / blk.x, (c.ny + blk.y - 1) / blk.y, c.nz);
+        k_rest_solid<Q, S><<<grd, blk, 0, c.stream>>>(static_cast<typename S::T*>(f), geom(c), c.links);
+        return cudaGetLastError();
+    });
 }
 
 // ---------------------------------------------------------------------------
