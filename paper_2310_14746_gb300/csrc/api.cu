@@ -28,10 +28,15 @@ int cuda_fail(cudaError_t e) {
         if (e_ != cudaSuccess) return cuda_fail(e_);  \
     } while (0)
 
-// Steps of the two step graphs: the long one while a run has as many left, the short one below.
-// Even: a graph returns the state to its starting layout. A replay costs about 3 us beside its kernels
-// (kernels chained, us per step, 8 / 16 / 32 / 64 steps: 32^3 2.31 / 2.05 / 2.01 / 1.95).
+// Steps of the two step graphs. Even: a graph returns the state to its starting layout. A replay
+// costs about 3 us beside its kernels (kernels chained, us per step, 8 / 16 / 32 / 64 steps: 32^3
+// 2.31 / 2.05 / 2.01 / 1.95), and capturing and instantiating a graph about 15 us and 3 us per step,
+// again after every change of a setting. So the long one is captured once kLongFrom steps have been
+// asked for with the present settings (a change of the force and 24 steps of 24^3: both graphs 125
+// us, the short one alone 91; and 96 steps: 255 either way), and the short one, for what the long one leaves, not before
+// kShortFrom.
 constexpr int kGraphSteps[] = {8, 16};
+constexpr long long kLongFrom = 96, kShortFrom = 512;
 // Runs of a small lattice that one resident launch takes: below kResidentMin the launch and its
 // loads and stores (about 5 us) cost more than single steps; kResidentMax bounds one launch to
 // about a millisecond or two.
@@ -75,6 +80,7 @@ struct hlbm_lattice {
     double* out8_host = nullptr;
     cudaGraphExec_t gexec[2] = {};  // of kGraphSteps
     bool graph_valid[2] = {};       // captured with the present settings?
+    long long graph_steps = 0;      // steps asked of hlbm_step with the present settings
     int chaining = CHAIN_NONE;      // of the steps that are launched next
     cudaGraphExec_t series_exec = nullptr;  // kSeriesSamples samples of hlbm_reduce_series
     int series_every = 0;                   // steps between its samples; 0: to be captured again
@@ -82,6 +88,7 @@ struct hlbm_lattice {
     cudaEvent_t series_ev[3] = {};
     void settings_changed() {
         graph_valid[0] = graph_valid[1] = false;
+        graph_steps = 0;
         series_every = 0;
     }
     int step_variant = HLBM_STEP_AUTO;
@@ -698,9 +705,12 @@ int hlbm_step(hlbm_t* h, long nsteps) {
         }
     }
     const bool two = left >= 4 && two_steps(h);
+    h->graph_steps += left;
+    const bool use_long = h->graph_valid[1] || h->graph_steps >= kLongFrom;
     while (left > 0) {
-        if (left >= kGraphSteps[0] && at_graph_origin(h)) {
-            const int k = left >= kGraphSteps[1];
+        const int k = use_long && left >= kGraphSteps[1];
+        const bool use = k || h->graph_valid[0] || !h->graph_valid[1] || h->graph_steps >= kShortFrom;
+        if (use && left >= kGraphSteps[0] && at_graph_origin(h)) {
             if (!h->graph_valid[k]) {
                 int rc = build_graph(h, k);
                 if (rc != HLBM_OK) return rc;
@@ -709,7 +719,7 @@ int hlbm_step(hlbm_t* h, long nsteps) {
             left -= kGraphSteps[k];
             h->step += kGraphSteps[k];
         } else {
-            const int n = two && left >= 4 && left < kGraphSteps[0] ? 4 : 1;
+            const int n = two && left >= 4 && (!use || left < kGraphSteps[0]) ? 4 : 1;
             int rc = steps_on(h, h->stream, n, two);
             if (rc != HLBM_OK) return rc;
             left -= n;
