@@ -35,9 +35,8 @@
 // Variants that were slower at 256^3: two larger blocks per SM with the whole
 // window in registers 340, one tensor-map box per direction 341, a bulk copy per row 386,
 // delay lines in registers 337, and every 16-bit variant (bound by instructions).
-#include <cmath>
-
 #include "k_step_pair.cuh"
+#include "step2_plan.h"
 
 namespace hlbm {
 
@@ -45,7 +44,7 @@ namespace {
 
 using L = Lat<19>;
 
-constexpr int kBlocksPerSM = 3;
+constexpr int kBlocksPerSM = kStep2BlocksPerSM;
 
 // Position of direction i within the directions of the same c_z, in index order, and
 // the first position of a c_z group in the staging buffer (up, flat, down).
@@ -234,38 +233,6 @@ k_step2(const float* __restrict__ fin, float* __restrict__ fout, const float* __
     }
 }
 
-// Tile and planes per block with the least time, in phases of one plane of the 32 x 7 tile (about
-// 1.75 us for a phase pair with every SM full): a block of zc planes runs zc + 2 planes of phase 1 and zc of
-// phase 2, and starts and ends with a wait; a plane of the 24 x 9 tile takes 0.945 of that; the
-// blocks of a single wave run in step and take 1.03; a last wave that is partly full saves a fifth of
-// what is missing. Two steps, 32 x 7 / 24 x 9, us: 128^3 88.7 / 94.6, 160^3 177 / 167, 240^3
-// 541 / 501, 256^3 617 / 615, 288^3 864 / 840. Over 60 lattices with two to four measured plans
-// each, the plan chosen here took 0.6 % more than the best of them. Slower: 16 x 14 (256^3 671),
-// and with two blocks per SM 48 x 7 (721) and 32 x 11 (651, though 163 at 160^3).
-struct Step2Plan {
-    bool wide;      // 32 x 7, else 24 x 9
-    int zc;
-    double useful;  // cells over the cells that the waves' blocks have room for
-};
-Step2Plan step2_plan(const LaunchCtx& c) {
-    constexpr int kSlots = kBlocksPerSM * 152;
-    Step2Plan best{true, c.nz, 0.0};
-    for (const bool wide : {true, false}) {
-        const int tx = wide ? 32 : 24, ty = wide ? 7 : 9;
-        const long long bxy = (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty);
-        for (int k = 1; k <= c.nz; ++k) {
-            const int zc = (c.nz + k - 1) / k, bz = (c.nz + zc - 1) / zc;
-            const double full = (double)(bxy * bz) / kSlots, waves = std::ceil(full);
-            const double turns = waves > 1.0 ? waves - 0.2 * (waves - full) : 1.03;
-            const double time = turns * (2.0 * zc + 3.0) * (wide ? 1.0 : 0.945);
-            const double useful = 2.0 * c.nx * c.ny * c.nz / (time * kSlots * 32 * 7);
-            if (useful > best.useful) best = {wide, zc, useful};
-            if (zc <= 8) break;
-        }
-    }
-    return best;
-}
-
 template <int FORM, int TX, int TY>
 cudaError_t step2_tile(const LaunchCtx& c, int zc, const void* fin, void* fout, const float* varpi) {
     using K = Tile<TX, TY>;
@@ -299,7 +266,8 @@ bool step2_applies(const LaunchCtx& c) {
         c.nx < 8 || c.ny < 4 || c.nz < 4 || 19 * n >= ((size_t)1 << 31) || n < 1500000)
         return false;
     const int form = step_form(c, 19);
-    return step2_plan(c).useful >= (form == FORM_SHIFT_FX ? 0.78 : (form == FORM_ANISO ? 0.86 : 0.83));
+    const double need = form == FORM_SHIFT_FX ? 0.78 : (form == FORM_ANISO ? 0.86 : 0.83);
+    return step2_plan(c, need).useful >= need;
 }
 
 cudaError_t launch_step2(const LaunchCtx& c, const void* fin, void* fout, const float* varpi) {
