@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <utility>
@@ -186,6 +187,14 @@ cudaError_t launch_fill_f32(float* v, size_t n, float value, cudaStream_t s);
 cudaError_t launch_fill_bytes0(void* p, size_t bytes, cudaStream_t s);
 
 size_t storage_bytes(int storage);
+
+// A yes or no about the current context (a context may be confined to a part of its device, so a
+// device's answer need not hold in it), asked when the context is not the one of the last answer.
+// `ask` returns 1 or 0, or -1 when it could not tell: that counts as no and is not remembered.
+struct ContextFact {
+    std::atomic<unsigned long long> known[64] = {};  // per device: context id * 2 + answer
+    bool get(int (*ask)());
+};
 
 // Memory kept between objects, in the current context (mem.cu). A pool belongs to one handle at
 // a time; every block taken from it is freed, and its streams are drained, before it is released.

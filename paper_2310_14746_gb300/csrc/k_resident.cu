@@ -10,8 +10,6 @@
 // neighbour's, with the periodic wrap, walls and obstacles folded in), so a
 // step is q loads, the collision and q local stores per cell, then one cluster
 // barrier. The collision is the one of the per-cell kernels: the same bits.
-#include <atomic>
-
 #include "k_step.cuh"
 
 namespace hlbm {
@@ -184,42 +182,35 @@ cudaError_t resident_q(const LaunchCtx& c, const ResidentPlan& p, void* f, const
 // take longer than the whole chip and a launch.
 size_t resident_cells_max(int q) { return (size_t)kBlocks * kMaxThreads * (q == 9 ? 2 : 1); }
 
-// Whether the device can run the largest cluster (16 blocks is beyond the portable
-// size: it needs sixteen free SMs behind one cluster scheduler); asked once per device.
-bool cluster_available() {
-    constexpr int kMaxDevices = 64;
-    static std::atomic<int> known[kMaxDevices];  // 0 not asked, 1 yes, 2 no
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
-    int k = known[dev].load(std::memory_order_relaxed);
-    if (k == 0) {
-        const auto kern = k_resident<19, StoreF32, FORM_SHIFT, 1>;
-        const int bytes = 2 * 19 * kMaxThreads * (int)sizeof(float);
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(kBlocks);
-        cfg.blockDim = dim3(kMaxThreads);
-        cfg.dynamicSmemBytes = bytes;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = kBlocks;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int n = 0;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-        if (e != cudaSuccess) (void)cudaGetLastError();
-        k = e == cudaSuccess && n >= 1 ? 1 : 2;
-        known[dev].store(k, std::memory_order_relaxed);
-    }
-    return k == 1;
+// Can the current context run the largest cluster (16 blocks is beyond the portable size: it
+// needs sixteen free SMs behind one cluster scheduler)?
+int ask_cluster() {
+    const auto kern = k_resident<19, StoreF32, FORM_SHIFT, 1>;
+    const int bytes = 2 * 19 * kMaxThreads * (int)sizeof(float);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kBlocks);
+    cfg.blockDim = dim3(kMaxThreads);
+    cfg.dynamicSmemBytes = bytes;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kBlocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    if (e == cudaSuccess) return n >= 1;
+    (void)cudaGetLastError();
+    return -1;
 }
+ContextFact g_cluster;
 
 }  // namespace
 
 bool resident_applies(const LaunchCtx& c) {
-    return c.variant == 0 && c.storage != 0 && (size_t)c.nx * c.ny * c.nz <= resident_cells_max(c.q) && cluster_available();
+    return c.variant == 0 && c.storage != 0 && (size_t)c.nx * c.ny * c.nz <= resident_cells_max(c.q) && g_cluster.get(ask_cluster);
 }
 
 cudaError_t launch_resident(const LaunchCtx& c, void* f, const float* varpi, int nsteps) {

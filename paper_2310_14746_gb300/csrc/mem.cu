@@ -32,6 +32,7 @@ namespace hlbm {
 namespace {
 
 constexpr int kMaxDevices = 64, kContexts = 4;
+static_assert(sizeof(ContextFact::known) / sizeof(ContextFact::known[0]) == kMaxDevices);
 // per context:
 constexpr size_t kKeepPools = 2, kKeepBytes = (size_t)512 << 20;  // at most 1.5 GiB stays mapped
 constexpr size_t kKeepPinned = (size_t)64 << 20;
@@ -145,6 +146,20 @@ cudaError_t create_pool(unsigned long long hold, cudaMemPool_t* pool) {
 }  // namespace
 
 // All functions here work in the current context.
+
+bool ContextFact::get(int (*ask)()) {
+    int device = -1;
+    if (cudaGetDevice(&device) != cudaSuccess) return false;
+    const unsigned long long id = context_id();
+    const bool remembers = id && device >= 0 && device < kMaxDevices;
+    if (remembers) {
+        const unsigned long long k = known[device].load(std::memory_order_relaxed);
+        if (k >> 1 == id) return k & 1;
+    }
+    const int yes = ask();
+    if (remembers && yes >= 0) known[device].store(id * 2 + yes, std::memory_order_relaxed);
+    return yes == 1;
+}
 
 void memory_give_back() {
     cudaMemPool_t pools[kKeepPools];

@@ -206,6 +206,28 @@ void no_host_memory() {
     expect(g_pools.size() == 1 && g_pinned.size() == 1, "the servers' pool and the slots stay, nothing else");
 }
 
+// A fact is asked once per context, of the context that is current, and an error is not remembered.
+int g_asked = 0, g_answer = 1;
+void context_facts() {
+    static ContextFact fact;
+    const auto ask = [] { return ++g_asked, g_answer; };
+    expect(fact.get(ask) && fact.get(ask) && g_asked == 1, "asked once");
+    g_context = 2;
+    g_answer = 0;
+    expect(!fact.get(ask) && !fact.get(ask) && g_asked == 2, "another context is asked, and has its own answer");
+    g_context = 1;
+    g_answer = 1;
+    expect(fact.get(ask), "the first context keeps its answer");
+    g_context = 3;
+    g_answer = -1;
+    expect(!fact.get(ask), "an error is a no");
+    g_answer = 1;
+    expect(fact.get(ask), "that is not remembered");
+    g_context = 0;
+    g_answer = 0;
+    expect(!fact.get(ask), "no context");
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -213,6 +235,7 @@ int main(int argc, char** argv) {
     if (!std::strcmp(name, "no_context_ids")) no_context_ids();
     else if (!std::strcmp(name, "several_contexts")) several_contexts();
     else if (!std::strcmp(name, "no_host_memory")) no_host_memory();
+    else if (!std::strcmp(name, "context_facts")) context_facts();
     else expect(false, "a case of this program");
     return g_failed;
 }

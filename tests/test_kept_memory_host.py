@@ -25,7 +25,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("case", ["no_context_ids", "several_contexts", "no_host_memory"])
+@pytest.mark.parametrize("case", ["no_context_ids", "several_contexts", "no_host_memory", "context_facts"])
 def test_kept_memory(program, case):
     r = subprocess.run([program, case], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stderr
