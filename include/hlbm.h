@@ -230,9 +230,20 @@ int hlbm_get_populations(hlbm_t* h, double* f, int on_device);
 /* ---- time stepping ----------------------------------------------------- */
 
 /* Advance nsteps >= 0 time steps (stream + collide, see above). Asynchronous.
- * Runs of at least 8 steps replay captured CUDA graphs of the step
- * sequence; shorter runs launch directly. */
+ * Three paths give the same bits with two-lattice streaming: a lattice of at
+ * most 8192 cells (D3Q19) or 16384 (D2Q9) in FP32, FP16 or BF16 storage runs 6
+ * and more steps in one launch, resident in shared memory; a periodic FP32
+ * D3Q19 lattice of at least 1.5 million cells with nx a multiple of 4, whose
+ * shape fills the GPU evenly, goes two steps per launch in runs of four; all
+ * others go one step per launch. The last two replay captured CUDA graphs of
+ * 8 and 16 steps in runs of at least 8 (a step or more launched singly where
+ * a run starts or ends between them). Only runs without a graph can be
+ * captured into a graph of the caller's. */
 int hlbm_step(hlbm_t* h, long nsteps);
+/* How many time steps the first launch of a run of nsteps advances with the
+ * present settings: 1, 2, or up to 1000 where the run is resident (no
+ * counterpart in the paper: for testing and measurement). */
+int hlbm_steps_per_launch(hlbm_t* h, long nsteps, long* steps);
 
 /* Steps taken since the last initialisation. */
 int hlbm_get_step(hlbm_t* h, long long* step);

@@ -132,6 +132,7 @@ SIGNATURES = {
     "hlbm_set_populations": (_i, [_vp, _vp, _i]),
     "hlbm_get_populations": (_i, [_vp, _vp, _i]),
     "hlbm_step": (_i, [_vp, ctypes.c_long]),
+    "hlbm_steps_per_launch": (_i, [_vp, ctypes.c_long, ctypes.POINTER(ctypes.c_long)]),
     "hlbm_get_step": (_i, [_vp, ctypes.POINTER(ctypes.c_longlong)]),
     "hlbm_moments": (_i, [_vp, _vp, _vp, _i]),
     "hlbm_moments_f64": (_i, [_vp, _vp, _vp, _i]),
@@ -306,6 +307,12 @@ def hlbm_get_populations(h, out):
 
 def hlbm_step(h, nsteps):
     _check(_lib().hlbm_step(h, int(nsteps)), "hlbm_step")
+
+
+def hlbm_steps_per_launch(h, nsteps):
+    n = ctypes.c_long()
+    _check(_lib().hlbm_steps_per_launch(h, int(nsteps), ctypes.byref(n)), "hlbm_steps_per_launch")
+    return n.value
 
 
 def hlbm_get_step(h):
@@ -529,6 +536,10 @@ class Lattice:
 
     def step(self, n=1):
         hlbm_step(self.h, n)
+
+    def steps_per_launch(self, nsteps):
+        """Time steps that the first launch of step(nsteps) advances (1, 2, or many: resident)."""
+        return hlbm_steps_per_launch(self.h, nsteps)
 
     @property
     def steps_taken(self):

@@ -33,8 +33,8 @@ int cuda_fail(cudaError_t e) {
 // 2.31 / 2.05 / 2.01 / 1.95), and capturing and instantiating a graph about 15 us and 3 us per step,
 // again after every change of a setting. So the long one is captured once kLongFrom steps have been
 // asked for with the present settings (a change of the force and 24 steps of 24^3: both graphs 125
-// us, the short one alone 91; and 96 steps: 255 either way), and the short one, for what the long one leaves, not before
-// kShortFrom.
+// us, the short one alone 91; and 100 steps: 254 to 258 either way), and the short one, for what the
+// long one leaves, not before kShortFrom.
 constexpr int kGraphSteps[] = {8, 16};
 constexpr long long kLongFrom = 96, kShortFrom = 512;
 // Runs of a small lattice that one resident launch takes: below kResidentMin the launch and its
@@ -193,6 +193,9 @@ int step_once(hlbm_t* h, cudaStream_t s) {
     return HLBM_OK;
 }
 
+bool resident(const hlbm_t* h, long n) {
+    return h->pattern == HLBM_TWO_LATTICE && n >= kResidentMin && resident_applies(h->ctx(h->stream));
+}
 bool two_steps(const hlbm_t* h) { return h->pattern == HLBM_TWO_LATTICE && step2_applies(h->ctx(h->stream)); }
 
 // n steps on `s`, where `two` in pairs of two-step launches: four steps then end in the buffer
@@ -696,7 +699,7 @@ int hlbm_step(hlbm_t* h, long nsteps) {
     if (!h || nsteps < 0) return HLBM_ERR_INVALID_ARG;
     DeviceGuard g(h->device);
     long left = nsteps;
-    if (h->pattern == HLBM_TWO_LATTICE && left >= kResidentMin && resident_applies(h->ctx(h->stream))) {
+    if (resident(h, left)) {
         while (left >= kResidentMin) {
             const long n = left < kResidentMax ? left : kResidentMax;
             HLBM_CUDA(launch_resident(h->ctx(h->stream), h->state(), h->varpi, (int)n));
@@ -726,6 +729,14 @@ int hlbm_step(hlbm_t* h, long nsteps) {
             h->step += n;
         }
     }
+    return HLBM_OK;
+}
+
+int hlbm_steps_per_launch(hlbm_t* h, long nsteps, long* steps) {
+    if (!h || !steps || nsteps < 0) return HLBM_ERR_INVALID_ARG;
+    DeviceGuard g(h->device);
+    if (resident(h, nsteps)) *steps = nsteps < kResidentMax ? nsteps : kResidentMax;
+    else *steps = nsteps >= 4 && two_steps(h) ? 2 : 1;
     return HLBM_OK;
 }
 
