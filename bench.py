@@ -12,9 +12,9 @@ e2e   : the same metric through the C ABI with host buffers: per step the porosi
         is copied from pinned host memory (set_porosity), the lattice re-initialised,
         100 time steps run and the diagnostics read back to the host.
 roofline : the stream-collide kernel's algorithmic bytes (q*2*sizeof(T) + 4 per cell and
-        launch) over its average launch time, against the measured HBM copy bandwidth. A
-        launch of the FP32 two-lattice workloads advances two steps (steps_per_launch), so
-        its bytes per cell update are half of that.
+        launch) over its average launch time, against the measured HBM copy bandwidth. Where
+        a launch advances two steps (hlbm_steps_per_launch; the large FP32 two-lattice
+        workloads), its bytes per cell update are half of that; steps_per_launch is the mean.
 cpu_baseline : the FP64 CPU oracle timed on the host cores on a bounded sample (a few
         time steps of the same 256^3 workload).
 
@@ -82,30 +82,35 @@ KERNEL_SOURCES = {
 }
 
 
-def steps_per_launch(w):
-    """Time steps that one launch of the workload's step kernel advances: two for the periodic FP32
-    two-lattice cubes here, all larger than L2 (csrc/k_step2.cu), else one."""
-    return 2 if w["q"] == 19 and w["storage"] == "f32" and w["pattern"] == "two" else 1
+# the kernel that advances two steps per launch (FP32, two-lattice), and its traffic per launch by edge:
+# k_step2<shift-fx>, 256^3, mean of two launches (1442929664 + 1239572480 and 1437650944 + 1232098304 bytes)
+TWO_STEP_SOURCES = _COMMON_SOURCES + ("k_step_pair.cuh", "k_step2.cu", "step2_plan.h")
+TWO_STEP_TRAFFIC_BYTES = {256: {"bytes": 2676125696, "source_hash": "0000000000000000"}}
 
 
-def kernel_source_hash(kname):
+def step_launches(steps_per_launch, nsteps):
+    """Launches of a run of nsteps whose first launch advances steps_per_launch: two-step launches go in
+    pairs, and the last one to three steps single."""
+    return nsteps // 4 * 2 + nsteps % 4 if steps_per_launch == 2 else -(-nsteps // steps_per_launch)
+
+
+def kernel_source_hash(kname, two_steps=False):
     """sha256 (first 16 hex digits) over the sources of the step kernel `kname`
-    (stream_collide_d3q19_<storage>_<pattern>)."""
+    (stream_collide_d3q19_<storage>_<pattern>), or of the two-step kernel in its place."""
     import hashlib
-    storage = kname.split("_")[3]
     h = hashlib.sha256()
-    for name in KERNEL_SOURCES[storage]:
+    for name in TWO_STEP_SOURCES if two_steps else KERNEL_SOURCES[kname.split("_")[3]]:
         with open(os.path.join(ROOT, "paper_2310_14746_gb300", "csrc", name), "rb") as fh:
             h.update(name.encode() + b"\0" + fh.read())
     return h.hexdigest()[:16]
 
 
-def kernel_traffic(kname, n):
+def kernel_traffic(kname, n, two_steps=False):
     """(bytes per launch or None, note) for the kernel as it is now."""
-    e = KERNEL_TRAFFIC_BYTES.get((kname, n))
+    e = TWO_STEP_TRAFFIC_BYTES.get(n) if two_steps else KERNEL_TRAFFIC_BYTES.get((kname, n))
     if e is None:
         return None, "not captured"
-    if e["source_hash"] != kernel_source_hash(kname):
+    if e["source_hash"] != kernel_source_hash(kname, two_steps):
         return None, "stale: kernel sources changed since the capture"
     return e["bytes"], "ncu capture of these sources"
 
@@ -749,9 +754,10 @@ def run_gpu(args, w, rank, world, local_rank):
     lat.set_porosity(varpi_pinned.numpy())
     lat.init_equilibrium()
 
-    per_launch = steps_per_launch(w)
-    # stream-collide launches (two-step ones in pairs, the last one to three steps single) + 2 reduction kernels
-    launches_per_step = (inner if per_launch == 1 else inner // 4 * 2 + inner % 4) + 2
+    two_steps = lat.steps_per_launch(inner) == 2
+    step_kernels = step_launches(lat.steps_per_launch(inner), inner)
+    launches_per_step = step_kernels + 2  # + 2 reduction kernels
+    per_launch = inner / step_kernels
 
     def one_step(ev_a=None, ev_b=None):
         if ev_a is not None:
@@ -804,7 +810,7 @@ def run_gpu(args, w, rank, world, local_rank):
     achieved = bytes_per_lup * cells / (kern_ms * 1e-3) / 1e9
     peak, peak_kind = measured_hbm_peak()
     kname = "stream_collide_d%dq%d_%s_%s" % (3 if q == 19 else 2, q, w["storage"], w["pattern"])
-    traffic, traffic_note = kernel_traffic(kname, n)
+    traffic, traffic_note = kernel_traffic(kname, n, two_steps)
 
     aa = None
     if not args.no_legs and w["pattern"] == "two" and w["storage"] == "f32":
@@ -843,7 +849,7 @@ def run_gpu(args, w, rank, world, local_rank):
             "config": workload_config(w, inner, world),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic, "traffic_note": traffic_note,
-                         "kernel_source_hash": kernel_source_hash(kname), "peak_kind": peak_kind,
+                         "kernel_source_hash": kernel_source_hash(kname, two_steps), "peak_kind": peak_kind,
                          "kernel": kname, "kernel_ms": kern_ms * per_launch, "steps_per_launch": per_launch,
                          "bytes_per_lup": bytes_per_lup},
             "e2e": {"value": e2e_value, "unit": "MLUPS", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
