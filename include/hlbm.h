@@ -122,13 +122,14 @@ void hlbm_destroy(hlbm_t* h);
 
 /* Temporary device memory of the calls that need it (the checkpoints of
  * hlbm_adjoint_flux_grad, staging buffers of host-array I/O) comes, ordered on
- * the handle's stream, from a memory pool private to the handle, which keeps
- * the memory it has mapped for the next call instead of handing it back at
- * each synchronisation (re-mapping the 14.5 GB of checkpoints of a 128^3 x
+ * the handle's stream, from a memory pool that is the handle's own while it
+ * lives and serves a later handle afterwards (see hlbm_destroy). It keeps the
+ * memory it has mapped for the next call instead of handing it back at each
+ * synchronisation (re-mapping the 14.5 GB of checkpoints of a 128^3 x
  * 2000-step gradient took about 7 % of the call). This call waits for the
  * handle's stream and returns the pool's unused memory to the device, and with
- * it what is kept mapped for later handles and servers in the current context; the
- * next call that needs scratch maps it again. Not a paper operation (memory
+ * it what is kept mapped for later handles and servers in the current context;
+ * the next call that needs scratch maps it again. Not a paper operation (memory
  * management of this library). */
 int hlbm_release_scratch(hlbm_t* h);
 

@@ -5,15 +5,14 @@
 // steps, whose kernels run 1.6 ms): a design loop or a batch of small solves pays
 // that for every object. A handle therefore takes its scratch, and its lattice if
 // that is small, from a private stream-ordered pool, and a pool that is given back
-// is kept for the next handle on that device, trimmed to kKeepBytes; at most kKeepPools
-// are kept, the others are destroyed. Servers share one pool that
-// holds up to kKeepBytes unused (a slot's memory was mapped at each admission). Pinned
-// blocks are kept likewise, up to kKeepPinned bytes. A failed allocation first
-// returns what is kept. What is kept belongs to the context that was current when it was
-// allocated, and serves and is returned in that context only; up to kContexts contexts of a
-// device keep something, in any further one nothing is kept. Measured: gradient of a 48^3 box over
-// 90 steps through torch.autograd, handle included, 3.80 -> 2.10 ms; submitting a 96^3
-// request 1.2 -> 0.34 ms.
+// is kept for the next handle, trimmed to kKeepBytes; at most kKeepPools are kept, the
+// others are destroyed. Servers share one pool that holds up to kKeepBytes unused (a
+// slot's memory was mapped at each admission). Pinned blocks are kept likewise, up to
+// kKeepPinned bytes. A failed allocation first returns what is kept. What is kept belongs
+// to the context that was current when it was allocated, and serves and is returned in that
+// context only; up to kContexts contexts of a device keep something, a further one nothing.
+// Measured: gradient of a 48^3 box over 90 steps through torch.autograd, handle included,
+// 3.80 -> 2.10 ms; submitting a 96^3 request 1.2 -> 0.34 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
