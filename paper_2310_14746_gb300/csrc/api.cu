@@ -58,8 +58,8 @@ struct hlbm_lattice {
     int q = 19, nx = 0, ny = 0, nz = 0, storage = HLBM_F32, pattern = HLBM_TWO_LATTICE;
     int device = 0;
     cudaStream_t stream = nullptr;
-    cudaStream_t own_stream = nullptr;  // of the handle alone: graphs are captured there, and gradients run there
-    cudaEvent_t own_ev = nullptr;
+    cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
+    cudaEvent_t fork_ev = nullptr;      // where a gradient leaves the handle's stream
     double tau = 1.0;
     double F[3] = {0.0, 0.0, 0.0};
     int bc[3] = {HLBM_PERIODIC, HLBM_PERIODIC, HLBM_PERIODIC};
@@ -168,8 +168,8 @@ void free_all(hlbm_t* h) {
     for (cudaEvent_t e : h->series_ev)
         if (e) cudaEventDestroy(e);
     if (h->series_stream) cudaStreamDestroy(h->series_stream);
-    if (h->own_ev) cudaEventDestroy(h->own_ev);
-    if (h->own_stream) cudaStreamDestroy(h->own_stream);
+    if (h->fork_ev) cudaEventDestroy(h->fork_ev);
+    if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     void* const blocks[] = {h->buf[0], h->buf[1], h->varpi, h->u_prev, h->partials, h->out8};
     for (void* p : blocks)
         if (p && (!h->pooled || cudaFreeAsync(p, h->stream) != cudaSuccess)) cudaFree(p);
@@ -212,16 +212,16 @@ int steps_on(hlbm_t* h, cudaStream_t s, long n, bool two) {
 
 bool at_graph_origin(const hlbm_t* h) { return h->pattern == HLBM_TWO_LATTICE ? h->cur == 0 : h->aa_odd == 0; }
 
-// Capture what `body` launches on the handle's own stream, starting from the graph origin layout,
+// Capture what `body` launches on the handle's capture stream, starting from the graph origin layout,
 // which an even number of steps returns to.
 template <class Body>
 int capture(hlbm_t* h, cudaGraphExec_t* exec, Body&& body) {
-    if (!h->own_stream) HLBM_CUDA(cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking));
+    if (!h->cap_stream) HLBM_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     const int cur0 = h->cur, odd0 = h->aa_odd;
     cudaGraph_t graph = nullptr;
-    HLBM_CUDA(cudaStreamBeginCapture(h->own_stream, cudaStreamCaptureModeThreadLocal));
-    const int rc = body(h->own_stream);
-    cudaError_t e = cudaStreamEndCapture(h->own_stream, &graph);
+    HLBM_CUDA(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+    const int rc = body(h->cap_stream);
+    cudaError_t e = cudaStreamEndCapture(h->cap_stream, &graph);
     h->cur = cur0;
     h->aa_odd = odd0;
     if (rc != HLBM_OK) {
@@ -859,22 +859,20 @@ struct Scratch {
     }
 };
 
-// The handle's own stream for the length of a call, behind what its stream holds so far. Chained
-// kernels (launch_chained) must follow one another directly: on the caller's stream another thread,
-// with a handle of its own, can put a copy or a graph between two of them, and here nobody can.
+// A stream for the length of a call, behind what the handle's stream holds so far. Chained kernels
+// (launch_chained) must follow one another directly: on the caller's stream another thread, with
+// a handle of its own, can put a copy or a graph between two of them, and here nobody can.
 // Waited for at the latest when the call ends, before its scratch is given back.
 struct OwnStream {
-    hlbm_t* h;
-    explicit OwnStream(hlbm_t* hh) : h(hh) {}
+    cudaStream_t s = nullptr;
     ~OwnStream() {
-        if (h->own_stream) cudaStreamSynchronize(h->own_stream);
+        if (s) stream_release(s, cudaStreamSynchronize(s) == cudaSuccess);
     }
-    cudaError_t fork() {
-        cudaError_t e = cudaSuccess;
-        if (!h->own_stream) e = cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking);
-        if (e == cudaSuccess && !h->own_ev) e = cudaEventCreateWithFlags(&h->own_ev, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventRecord(h->own_ev, h->stream);
-        return e == cudaSuccess ? cudaStreamWaitEvent(h->own_stream, h->own_ev, 0) : e;
+    cudaError_t fork(hlbm_t* h) {
+        cudaError_t e = stream_acquire(&s);
+        if (e == cudaSuccess && !h->fork_ev) e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(h->fork_ev, h->stream);
+        return e == cudaSuccess ? cudaStreamWaitEvent(s, h->fork_ev, 0) : e;
     }
 };
 
@@ -927,9 +925,9 @@ int hlbm_adjoint_flux_grad(hlbm_t* h, long nsteps, int every, int plane_x, doubl
     HLBM_CUDA(sc.alloc((void**)&gacc, N * sizeof(float)));
     HLBM_CUDA(sc.alloc((void**)&jdev, sizeof(double)));
     if (h->pattern != HLBM_TWO_LATTICE) HLBM_CUDA(sc.alloc((void**)&tmp, (size_t)h->q * N * sizeof(double)));
-    OwnStream own(h);
-    HLBM_CUDA(own.fork());
-    c.stream = h->own_stream;
+    OwnStream own;
+    HLBM_CUDA(own.fork(h));
+    c.stream = own.s;
     int rc = copy_natural(h, c, snaps, tmp);
     if (rc != HLBM_OK) return rc;
 

@@ -204,6 +204,10 @@ cudaError_t pool_acquire(cudaMemPool_t* pool);
 void pool_release(cudaMemPool_t pool);
 // The servers' pool; where nothing is kept, a new one that the caller destroys (own).
 cudaError_t pool_shared(cudaMemPool_t* pool, bool* own);
+// A stream for the length of a call. Released with `idle` when it has been waited for, and not
+// when that failed (within a capture): it is then destroyed.
+cudaError_t stream_acquire(cudaStream_t* s);
+void stream_release(cudaStream_t s, bool idle);
 cudaError_t pool_alloc(cudaMemPool_t pool, void** p, size_t bytes, cudaStream_t s);
 cudaError_t device_malloc(void** p, size_t bytes);  // cudaMalloc, for blocks that no pool should hold
 void* pinned_acquire(size_t bytes, size_t* capacity);  // null: out of memory

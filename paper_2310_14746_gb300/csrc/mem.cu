@@ -11,6 +11,9 @@
 // kKeepPinned bytes. A failed allocation first returns what is kept. What is kept belongs
 // to the context that was current when it was allocated, and serves and is returned in that
 // context only; up to kContexts contexts of a device keep something, a further one nothing.
+// Streams for the length of a call are kept too: a stream created, used and destroyed for each
+// gradient made graphs with branches 4 % slower for the rest of the process (series of 200 samples
+// of 64^3 2475 -> 2568 us), with a kept one they are not.
 // Measured: gradient of a 48^3 box over 90 steps through torch.autograd, handle included,
 // 3.80 -> 2.10 ms; submitting a 96^3 request 1.2 -> 0.34 ms.
 #include <cuda_runtime.h>
@@ -35,16 +38,19 @@ static_assert(sizeof(ContextFact::known) / sizeof(ContextFact::known[0]) == kMax
 // per context:
 constexpr size_t kKeepPools = 2, kKeepBytes = (size_t)512 << 20;  // at most 1.5 GiB stays mapped
 constexpr size_t kKeepPinned = (size_t)64 << 20;
+constexpr size_t kKeepStreams = 4;
 constexpr size_t kSlotBytes = 64, kSlots = 256;  // small pinned results (one page-locked block)
 
 struct Kept {
     unsigned long long context = 0;  // id of the context that all of this belongs to; 0: a free record
     cudaMemPool_t pools[kKeepPools] = {};
     size_t npools = 0;
+    cudaStream_t streams[kKeepStreams] = {};
+    size_t nstreams = 0;
     cudaMemPool_t shared = nullptr;
     std::multimap<size_t, void*> pinned;  // capacity -> block
     size_t pinned_bytes = 0;
-    std::set<void*> held;  // pools and pinned blocks that objects have
+    std::set<void*> held;  // pools, pinned blocks and streams that objects have
     char* slots = nullptr;
     std::vector<int> free_slots;
 };
@@ -86,6 +92,8 @@ bool has_memory(Fn&& fn) {
 // ends), and a record stays its context's: an object may be released with another one current.
 struct Records {
     Kept of[kMaxDevices][kContexts];
+    Kept* used[kMaxDevices * kContexts] = {};  // those with a context (walking all of them costs 25 us)
+    int nused = 0;
 };
 Records* records() {  // null: out of host memory
     static Records* all = nullptr;
@@ -105,21 +113,21 @@ Kept* kept() {
         if (k.context) continue;
         if (!has_memory([&] { k.free_slots.reserve(kSlots); })) return nullptr;
         k.context = id;
+        all->used[all->nused++] = &k;
         return &k;
     }
     return nullptr;
 }
 
-// The record that a pool or pinned block is held under, which it is taken off; null: none.
+// The record that a pool, pinned block or stream is held under, which it is taken off; null: none.
 Kept* holder(void* p) {
-    if (Records* const all = records())
-        for (auto& device : all->of)
-            for (Kept& k : device)
-                if (k.held.erase(p)) return &k;
+    Records* const all = records();
+    for (int i = 0; all && i < all->nused; ++i)
+        if (all->used[i]->held.erase(p)) return all->used[i];
     return nullptr;
 }
 
-// Holds a new pool or pinned block under the current context.
+// Holds a new pool, pinned block or stream under the current context.
 void hold(void* p) {
     holder(p);  // a context that is gone may have had one at this address
     if (Kept* const k = kept()) has_memory([&] { k->held.insert(p); });
@@ -230,6 +238,38 @@ void pool_release(cudaMemPool_t pool) {
     cudaMemPoolDestroy(pool);
 }
 
+cudaError_t stream_acquire(cudaStream_t* s) {
+    {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        Kept* const k = kept();
+        if (k && k->nstreams) {
+            *s = k->streams[--k->nstreams];
+            has_memory([&] { k->held.insert(*s); });
+            return cudaSuccess;
+        }
+    }
+    const cudaError_t e = cudaStreamCreateWithFlags(s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) {
+        *s = nullptr;
+        return e;
+    }
+    std::lock_guard<std::mutex> lk(kept_mutex());
+    hold(*s);
+    return cudaSuccess;
+}
+
+void stream_release(cudaStream_t s, bool idle) {
+    {
+        std::lock_guard<std::mutex> lk(kept_mutex());
+        Kept* const k = holder(s);
+        if (idle && k && k->nstreams < kKeepStreams) {
+            k->streams[k->nstreams++] = s;
+            return;
+        }
+    }
+    cudaStreamDestroy(s);
+}
+
 cudaError_t pool_alloc(cudaMemPool_t pool, void** p, size_t bytes, cudaStream_t s) {
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaErrorMemoryAllocation) {
@@ -322,12 +362,13 @@ void slot_release(double* p) {
     {
         std::lock_guard<std::mutex> lk(kept_mutex());
         Records* const all = records();
-        for (int d = 0; all && d < kMaxDevices; ++d)
-            for (Kept& k : all->of[d])
-                if (k.slots && c >= k.slots && c < k.slots + kSlotBytes * kSlots) {  // never freed: others use the block
-                    k.free_slots.push_back((int)((c - k.slots) / kSlotBytes));
-                    return;
-                }
+        for (int i = 0; all && i < all->nused; ++i) {
+            Kept& k = *all->used[i];
+            if (k.slots && c >= k.slots && c < k.slots + kSlotBytes * kSlots) {  // never freed: others use the block
+                k.free_slots.push_back((int)((c - k.slots) / kSlotBytes));
+                return;
+            }
+        }
     }
     cudaFreeHost(p);
 }

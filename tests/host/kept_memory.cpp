@@ -97,6 +97,11 @@ cudaError_t cudaMemPoolDestroy(cudaMemPool_t p) {
     expect(g_pools.erase(p) == 1, "only an existing pool is destroyed");
     return cudaSuccess;
 }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
+    *s = reinterpret_cast<cudaStream_t>(g_next_pool += 16);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t p, size_t) {
     expect(g_pools.count(p) == 1, "only an existing pool is trimmed");
@@ -170,6 +175,21 @@ void several_contexts() {
     void* const p1 = pinned_acquire(1000, &ca);
     void* const p2 = pinned_acquire(1000, &cb);
     expect((p1 == pa && p2 == pb) || (p1 == pb && p2 == pa), "blocks go back to the context that they come from");
+
+    cudaStream_t s1 = nullptr, s2 = nullptr, s3 = nullptr;
+    stream_acquire(&s1);
+    stream_acquire(&s2);
+    expect(s1 && s2 && s1 != s2, "a stream for each call");
+    stream_release(s2, false);
+    g_context = 2;
+    stream_release(s1, true);
+    stream_acquire(&s3);
+    expect(s3 != s1 && s3 != s2, "a stream of the second context");
+    g_context = 1;
+    stream_acquire(&s2);
+    expect(s1 == s2, "an idle stream of the first context serves again");
+    stream_release(s2, true);
+    stream_release(s3, true);
 
     for (g_context = 3; g_context < 10; ++g_context) {  // more contexts than are kept for
         cudaMemPool_t p = nullptr;

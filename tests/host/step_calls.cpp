@@ -96,6 +96,8 @@ namespace hlbm {
 bool pool_keeps(size_t) { return true; }
 cudaError_t pool_acquire(cudaMemPool_t* p) { return *p = fresh<cudaMemPool_t>(), cudaSuccess; }
 void pool_release(cudaMemPool_t) {}
+cudaError_t stream_acquire(cudaStream_t* s) { return cudaStreamCreateWithFlags(s, 0); }
+void stream_release(cudaStream_t, bool) {}
 cudaError_t pool_alloc(cudaMemPool_t, void** p, size_t n, cudaStream_t) { return allocate(p, n); }
 cudaError_t device_malloc(void** p, size_t n) { return allocate(p, n); }
 double* slot_acquire() { return static_cast<double*>(std::malloc(64)); }
