@@ -56,20 +56,21 @@ FALLBACK_HBM_GBS = 6800.0
 # since, the bench reports traffic as null instead of a stale figure.
 KERNEL_TRAFFIC_BYTES = {
     # k_step<19, StoreF32, periodic, two-lattice, int, shift-fx>, 256^3: mean of two launches
-    # (1342250752 + 1228698112 and 1342237696 + 1217931008 bytes)
+    # (1342250752 + 1228698112 and 1342237696 + 1217931008 bytes), before the workload took two steps
+    # per launch (TWO_STEP_TRAFFIC_BYTES)
     ("stream_collide_d3q19_f32_two", 256): {"bytes": 2565558784, "source_hash": "76d4a47919d1105a"},
     # k_step<19, StoreF32, periodic, AA even / AA odd, int, shift-fx>, 256^3: mean of the even
-    # (1342405120 + 1216537856) and odd (1342217728 + 1214018048 bytes) launch of one capture
-    ("stream_collide_d3q19_f32_aa", 256): {"bytes": 2557589376, "source_hash": "1773fb175a24e720"},
+    # (1342199296 + 1216580864) and odd (1342235136 + 1214034176 bytes) launch of one capture
+    ("stream_collide_d3q19_f32_aa", 256): {"bytes": 2557524736, "source_hash": "fb226315581ab47b"},
     # k_step_pair<19, StoreF16, shift-fx, two-lattice>, 384^3 Boolean sphere matrix: mean of two launches
-    # (2378278656 + 2107357184 and 2378211072 + 2106170112 bytes)
-    ("stream_collide_d3q19_f16_two", 384): {"bytes": 4485008512, "source_hash": "59ee95aa12972e25"},
+    # (2378226688 + 2107194880 and 2378233088 + 2106194176 bytes)
+    ("stream_collide_d3q19_f16_two", 384): {"bytes": 4484924416, "source_hash": "3f47838038820ae6"},
     # k_step_pair<19, StoreBF16, shift-fx, two-lattice> (56 registers), 384^3 Boolean sphere matrix: mean of
-    # two launches (2378226176 + 2104031232 and 2378216704 + 2103352064 bytes)
-    ("stream_collide_d3q19_bf16_two", 384): {"bytes": 4481913088, "source_hash": "e6debcdf9dc15415"},
+    # two launches (2378240256 + 2103948800 and 2378222592 + 2103593472 bytes)
+    ("stream_collide_d3q19_bf16_two", 384): {"bytes": 4482002560, "source_hash": "756b2001393ed6ce"},
     # k_step_pair<19, StoreF16, shift-fx, AA even / AA odd>, 384^3 Boolean sphere matrix: mean of an
-    # even (2378207744 + 2097896192) and an odd (2378275584 + 2150258944 bytes) launch
-    ("stream_collide_d3q19_f16_aa", 384): {"bytes": 4502319232, "source_hash": "59ee95aa12972e25"},
+    # even (2378207232 + 2098303232) and an odd (2378458368 + 2149939968 bytes) launch
+    ("stream_collide_d3q19_f16_aa", 384): {"bytes": 4502454400, "source_hash": "3f47838038820ae6"},
 }
 
 # the sources each step kernel is compiled from (csrc/)
@@ -83,9 +84,9 @@ KERNEL_SOURCES = {
 
 
 # the kernel that advances two steps per launch (FP32, two-lattice), and its traffic per launch by edge:
-# k_step2<shift-fx>, 256^3, mean of two launches (1442929664 + 1239572480 and 1437650944 + 1232098304 bytes)
+# k_step2<shift-fx>, 256^3, mean of two launches (1433926912 + 1238616320 and 1437454336 + 1232751616 bytes)
 TWO_STEP_SOURCES = _COMMON_SOURCES + ("k_step_pair.cuh", "k_step2.cu", "step2_plan.h")
-TWO_STEP_TRAFFIC_BYTES = {256: {"bytes": 2676125696, "source_hash": "0000000000000000"}}
+TWO_STEP_TRAFFIC_BYTES = {256: {"bytes": 2671374592, "source_hash": "17263a81ef5017ed"}}
 
 
 def step_launches(steps_per_launch, nsteps):
