@@ -442,11 +442,19 @@ def aa_leg(args, w, field, stream):
                 workload="as the benchmark workload, in-place AA streaming (one population copy)")
 
 
+def adjoint_forward_launches(nsteps, every, two_steps):
+    """Step launches of a gradient's forward sweep (single steps in the last segment) and of the segments
+    that its reverse sweep recomputes."""
+    kept = (nsteps - 1) // every
+    sweep = kept * (every // 2 + every % 2 if two_steps else every) + nsteps - kept * every
+    return sweep + kept * (every - 1)
+
+
 def adjoint_leg(n=128, nsteps=2000, every=45, period=32, ratio=0.3, tau=0.6, F=(1e-6, 0.0, 0.0)):
     """Gradient of the outflow flux w.r.t. varpi on the adjoint workload (128^3 regular spheres,
     2000 steps, state kept every 45 steps): wall time of the whole call and its algorithmic
-    bytes: 156 per cell and forward launch (two steps each where no state in between is kept, single
-    ones in the last segment and when a segment is recomputed), 240 per cell and reverse step."""
+    bytes: 156 per cell and forward launch (on lattices that take two steps per launch, two steps each
+    where no state in between is kept), 240 per cell and reverse step."""
     import torch
     import paper_2310_14746_gb300 as hb
     from paper_2310_14746_gb300 import inputs
@@ -464,11 +472,10 @@ def adjoint_leg(n=128, nsteps=2000, every=45, period=32, ratio=0.3, tau=0.6, F=(
     J, _ = lat.adjoint_flux_grad(nsteps, every, n - 1, grad)
     torch.cuda.synchronize()
     dt = time.perf_counter() - t0
+    launches = adjoint_forward_launches(nsteps, every, lat.steps_per_launch(4) == 2)
     lat.close()
     cells = n ** 3
-    nsnap = (nsteps - 1) // every + 1
-    forward = (nsnap - 1) * (every // 2 + every % 2) + nsteps - (nsnap - 1) * every
-    algo = cells * ((forward + (nsnap - 1) * (every - 1)) * 156 + nsteps * 240)
+    algo = cells * (launches * 156 + nsteps * 240)
     peak, kind = measured_hbm_peak()
     return {"workload": "D3Q19 %d^3 regular spheres (period %d, r = %.1f P), %d steps, checkpoint every %d"
                         % (n, period, ratio, nsteps, every),

@@ -17,6 +17,13 @@ def test_launches_of_a_run(per_launch, nsteps, launches):
     assert bench.step_launches(per_launch, nsteps) == launches
 
 
+@pytest.mark.parametrize("nsteps,every,single,pairs", [(9, 4, 9 + 6, 2 + 2 + 1 + 6), (8, 4, 8 + 3, 2 + 4 + 3), (13, 5, 13 + 8, 3 + 3 + 3 + 8),
+                                                       (7, 20, 7, 7), (2000, 45, 2000 + 44 * 44, 44 * 23 + 20 + 44 * 44)])
+def test_launches_of_a_gradient(nsteps, every, single, pairs):
+    assert bench.adjoint_forward_launches(nsteps, every, False) == single
+    assert bench.adjoint_forward_launches(nsteps, every, True) == pairs
+
+
 def test_two_step_sources_and_traffic(monkeypatch):
     kname = "stream_collide_d3q19_f32_two"
     assert {"k_step2.cu", "step2_plan.h", "k_step_pair.cuh", "lattice.cuh"} <= set(bench.TWO_STEP_SOURCES)
